@@ -299,17 +299,17 @@ int mbl_lobpcg_solve_noalloc(const mbl_chain *chain, double sigma, const mbl_lob
  * independent levels of concurrency): nprob problems, any mix of L and fields, solved
  * with the same opts.  The workspace holds nstreams lanes; each lane solves one problem at
  * a time, and all lanes advance in lock step on `stream`, one LOBPCG iteration per round:
- * the steps before and after the preconditioner are enqueued lane by lane, and each of the
- * pcg_iters PCG steps of all advancing lanes runs as three launches over a table of the
- * lanes (so a round issues about 40 launches per lane plus 3 per PCG step, not 3 per PCG
- * step per lane).  When a lane's problem converges (or reaches max_iter) its results are
+ * the steps before and after the preconditioner are enqueued lane by lane, and the
+ * pcg_iters PCG steps of all advancing lanes run in cooperative launches of up to 64 steps,
+ * every lane on its own share of the SMs.  When a lane's problem converges (or reaches max_iter) its results are
  * written and it takes the next problem.  The host synchronises `stream` once per round
  * to read the lanes' status words.  With opts->use_graph, each lane's steps before and
  * after the preconditioner are captured once per problem as two small CUDA graphs and
  * replayed every round; opts->timing is ignored (use_graph = 0 with timing = 1 is
  * MBL_ERR_ARG).  Every problem's results equal the single-problem solve's to within
- * rounding (the PCG of a lane runs the same arithmetic in a batched launch; widths k other
- * than 8, 16, 32, 64 run each lane's own PCG launches and then equal them exactly).
+ * rounding (the PCG of a lane runs the same arithmetic on fewer SMs; widths k other than 8,
+ * 16, 32, 64, and lanes whose four PCG vectors exceed 100 MB, run each lane's own PCG
+ * launches and then equal them exactly).
  *   sigmas:   nprob shifts, or NULL: sigma_i = (E_min + E_max)/2 of problem i from
  *             the Lanczos bounds of mbl_spectrum_bounds (tolerance 1e-7, at most 1000
  *             steps, started from column 0 of its X0 block), found before the solves by

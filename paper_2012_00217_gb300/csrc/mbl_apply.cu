@@ -2062,229 +2062,667 @@ __global__ void __launch_bounds__(kThreads) k_pcg_update(uint32_t n, const T *__
 }
 
 // ---------------------------------------------------------------------------------
-// Batched PCG step (Sec. 3.1: realizations are independent): one launch covers the PCG
-// phase of many problems ("lanes"), each with its own chain, sector size, tile width,
-// vectors and per-column scalars, read from a table in device memory.  A lane's work
-// items are those of the persistent tiled product (a chunk of rows of one tile); the
-// items of all lanes form rounds of kWarps items, lane after lane, and each block takes a
-// contiguous run of rounds, so a block meets few lanes and rebuilds its shared tables
-// (chain constants, field tables) only when the lane changes.  Each round's column
-// partials (t.t or r.M^-1 r, compensated FP32 pairs in FP32) go to the lane's partials
-// by round; the block that completes a lane's last round sums them in round order and
-// finishes alpha or beta exactly as the single-problem launches do, so the results do not
-// depend on which block ran which round.  The row pass is the shared tile_row_pass.
+// Resident PCG: all the PCG steps of one or several problems ("lanes") in one cooperative
+// launch.  One block of 768 threads per SM serves one lane for the whole launch, so the
+// chain tables are built once, the small scalars of the recurrence live in shared memory,
+// and the phases of a step (t = (H - sigma)p with t.t; q = (H - sigma)t with r -= alpha q
+// and r.(M^-1 r); w += alpha p, p = M^-1 r + beta p) are separated by barriers among the
+// lane's blocks instead of by launches.
+//
+// What bounded the three launches of a step that this replaces: every launch paid its start,
+// its table set-up and a serial sum over the blocks' partials in its last block (33 us a
+// step at L = 12, k = 8, where the work itself is nothing), and the tiles, of 1 to C(B, B/2)
+// rows, fell on the blocks as their numbers came.  Here the work of a phase is split evenly:
+// the tiles are taken in order of falling size, whole by groups of 256 threads that go
+// through that order there and back (staged), or cut into row chunks dealt out to the warps.
+// Every block sums all partials of its lane itself, in a fixed order, right after the
+// barrier.  Measured (GB300, us a step, three launches -> resident):
+//   FP32  L = 12, k = 8: 32.8 -> 13.9;  14, 16: 35.9 -> 15.7;  16, 16: 40.3 -> 16.9;
+//         16, 64: 60.5 -> 22.3;  18, 32: 53.1 -> 31.0;  20, 32: 97.4 -> 83.8
+//   FP64  L = 14, k = 16: 118 -> 44.7;  18, 32: 236 -> 169
+// At L = 20, k = 32 the phases take about 22, 27 and 13 us of L2 traffic and the three
+// barriers with their sums the rest.  Beyond L2 (a lane's four vectors above 100 MB) the
+// launches are as fast or faster (L = 20, k = 64: 185 against 190 us; L = 22, k = 32: 301
+// against 404 us) and stay.
+//
+// A lane's blocks wait for one another, so the launch is cooperative.  Every wait is
+// bounded; on a time-out the lane's fail word is set, its blocks leave, and each writes
+// NaN into w, which the solver reports as MBL_ERR_NUMERIC.
 
+constexpr int kRunThreads = 768;
+constexpr int kRunWarps = kRunThreads / 32;
+constexpr int kRunSubs = kRunThreads / kThreads;  // staging groups of 256 threads
+constexpr int kRunJobs = 48;                      // cached tile jobs of a block
+constexpr int kRunSlots = 21;                     // 16-byte slots of tensor memory a thread has
+constexpr int kRunMaxBlocks = 160;                // blocks of a lane: five partials per lane of a warp
+constexpr int kRunStageBytes = 252 * 128;         // largest staged tile (C(10, 5) rows of 128 bytes); one per group
+constexpr long long kLaneWaitCycles = 10000000000ll;  // ~5 s at 2 GHz
 
-// Last lane whose first round (or row) is <= x: lanes are ordered by both.
-__device__ __forceinline__ int lane_of(const PcgLane *__restrict__ lanes, int nlanes, uint32_t x, bool by_row)
-{
-    int lo = 0, hi = nlanes - 1;
-    while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        const uint32_t v = by_row ? __ldg(&lanes[mid].row0) : __ldg(&lanes[mid].round0);
-        if (v <= x) lo = mid;
-        else hi = mid - 1;
+// Bytes of a row per lane of a warp: what the plain products use by default.
+__host__ __device__ constexpr int run_lane_bytes(int K, size_t es) { return (es == 8 && K * es >= 128) ? 64 : 32; }
+
+// A sum in the working precision of the reductions: a compensated pair in FP32, a double in
+// FP64.  Adding two of them gives the same result whichever comes first.
+template <typename T>
+struct ColSum;
+template <>
+struct ColSum<float> {
+    float s, e;
+    ColSum() = default;
+    __device__ __forceinline__ ColSum(float x, float y = 0.0f) : s(x), e(y) {}
+    __device__ __forceinline__ ColSum operator+(const ColSum &o) const
+    {
+        float hi, err;
+        two_sum(s, o.s, hi, err);
+        return ColSum(hi, (e + o.e) + err);
     }
-    return lo;
+    __device__ __forceinline__ ColSum shfl(int off) const
+    {
+        return ColSum(__shfl_xor_sync(0xffffffffu, s, off), __shfl_xor_sync(0xffffffffu, e, off));
+    }
+    // the value in FP64, and the pair nearest to one
+    __device__ __forceinline__ double value() const { return (double)s + (double)e; }
+    __device__ __forceinline__ static ColSum of(double v)
+    {
+        const float hi = (float)v;
+        return ColSum(hi, (float)(v - (double)hi));
+    }
+    __device__ __forceinline__ bool positive() const { return s > 0.0f && isfinite(s) && isfinite(e); }
+    __device__ __forceinline__ bool finite() const { return isfinite(s) && isfinite(e); }
+    // (s + e) / (d.s + d.e) in FP32: the quotient of the leading parts and one correction by
+    // the remainder, which the fma gives exactly; within an ulp of the rounded FP64 quotient
+    __device__ __forceinline__ float over(const ColSum &d) const
+    {
+        const float q = s / d.s;
+        const float r = fmaf(-q, d.s, s) + (e - q * d.e);
+        return q + r / d.s;
+    }
+    __device__ __forceinline__ void store(double *p) const { *reinterpret_cast<float2 *>(p) = make_float2(s, e); }
+    __device__ __forceinline__ static ColSum load(const double *p)
+    {
+        const float2 v = __ldcg(reinterpret_cast<const float2 *>(p));
+        return ColSum(v.x, v.y);
+    }
+};
+template <>
+struct ColSum<double> {
+    double s;
+    ColSum() = default;
+    __device__ __forceinline__ ColSum(double x) : s(x) {}
+    __device__ __forceinline__ ColSum operator+(const ColSum &o) const { return ColSum(s + o.s); }
+    __device__ __forceinline__ ColSum shfl(int off) const { return ColSum(__shfl_xor_sync(0xffffffffu, s, off)); }
+    __device__ __forceinline__ double value() const { return s; }
+    __device__ __forceinline__ static ColSum of(double v) { return ColSum(v); }
+    __device__ __forceinline__ bool positive() const { return s > 0.0 && isfinite(s); }
+    __device__ __forceinline__ bool finite() const { return isfinite(s); }
+    __device__ __forceinline__ double over(const ColSum &d) const { return s / d.s; }
+    __device__ __forceinline__ void store(double *p) const { *p = s; }
+    __device__ __forceinline__ static ColSum load(const double *p) { return ColSum(__ldcg(p)); }
+};
+
+// One unit of product work: rows [jb, je) of tile t.
+template <typename T>
+struct TileJob {
+    TileMeta<T> meta;
+    uint32_t t, jb, je;
+    int p;
+};
+
+template <typename T>
+struct RunShared {
+    uint32_t binom[kBinomDim * kBinomDim];
+    T tab[1024];
+    T red[kRunWarps][64];
+    TileJob<T> jobs[kRunJobs];
+    T alpha[64], beta[64];
+    ColSum<T> rz[64], tot[64];
+    int active[64];
+    uint32_t spref[kLowMaxB + 2];
+    uint32_t cls_item[kLowMaxB + 2];  // first item of each class of tiles, in falling size
+    int cls_p[kLowMaxB + 1], ncls;
+    PcgLane lane;
+    int ok;
+    uint32_t tmem;
+    __align__(8) uint64_t mbar[kRunSubs];
+    unsigned parity[kRunWarps];  // of the waits on mbar, per warp
+};
+
+// The block's state, at the start of its dynamic shared memory (the staged tiles follow),
+// so that the phases can be functions with registers of their own: inlined into one
+// kernel they spilled 0.5 to 1.9 KB a thread.
+template <typename T>
+__device__ __forceinline__ RunShared<T> &run_shared()
+{
+    extern __shared__ __align__(128) unsigned char run_raw[];
+    return *reinterpret_cast<RunShared<T> *>(run_raw);
 }
 
-template <typename T, int K, int MODE, int LB>
-__global__ void __launch_bounds__(kThreads, MBL_TILED_MIN_BLOCKS)
-    k_pcg_batch(const PcgLane *__restrict__ lanes, int nlanes, uint32_t total_rounds)
+template <typename T>
+__host__ __device__ constexpr size_t run_stage_offset()
 {
-    using Lay = WideRowLayout<T, K, LB>;
-    constexpr int V = Lay::V, G = Lay::G, RPW = 32 / G, CH = Lay::CH;
+    return (sizeof(RunShared<T>) + 127) / 128 * 128;
+}
+
+template <typename T>
+__device__ __forceinline__ T *as_global(void *p)
+{
+    T *q = reinterpret_cast<T *>(p);
+    __builtin_assume(__isGlobal(q));
+    return q;
+}
+
+__device__ __forceinline__ unsigned ld_relaxed(const unsigned *p)
+{
+    unsigned v;
+    asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+
+__device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.async;" ::: "memory"); }
+
+// All blocks of the lane have arrived `target` times in all.  false: a wait ran out.
+template <bool ASYNC, typename T>
+__device__ __forceinline__ bool lane_barrier(RunShared<T> &sm, unsigned &target)
+{
+    // the next phase may read by bulk copies what this one wrote by ordinary stores
+    if (ASYNC) fence_proxy_async();
+    __syncthreads();
+    const unsigned nb = sm.lane.nblocks;
+    if (nb == 1) return true;
+    target += nb;
+    if (threadIdx.x == 0) {
+        unsigned *bar = sm.lane.counter + 1;
+        const unsigned *fail = sm.lane.counter + 3;
+        // release: the block's stores of this phase come first; acquire: after the last arrival
+        asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(bar) : "memory");
+        int ok = 1;
+        const long long t0 = clock64();
+        for (unsigned polls = 1; ld_relaxed(bar) < target; ++polls) {
+            if (polls % 256u) continue;
+            if (ld_relaxed(fail)) ok = 0;
+            else if (clock64() - t0 > kLaneWaitCycles) {
+                atomicExch(sm.lane.counter + 3, 1u);
+                ok = 0;
+            }
+            if (!ok) break;
+        }
+        asm volatile("fence.acq_rel.gpu;" ::: "memory");
+        sm.ok = ok;
+    }
+    __syncthreads();
+    return sm.ok != 0;
+}
+
+// Column sums over the lane's blocks: the warps' sums sm.red -> sm.tot[K], the same in every
+// block.  buf: K x nblocks partials.  These few thousand cycles are paid twice a step with
+// the chip idle, so every stage is a tree: eight threads a column over the warps, a warp a
+// column over the blocks.  In FP32 neither they nor the scalars that follow touch the FP64
+// pipe, where one warp's instruction takes 64 cycles however few of its lanes are active.
+template <typename T, int K, bool ASYNC>
+__device__ __forceinline__ bool lane_column_sums(double *buf, unsigned &target)
+{
+    RunShared<T> &sm = run_shared<T>();
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int nb = (int)sm.lane.nblocks, bl = (int)(blockIdx.x - sm.lane.block0);
+    static_assert(kRunWarps == 24 && 8 * K <= kRunThreads, "three warps' sums for each of eight threads");
+    __syncthreads();
+    if (threadIdx.x < 8 * K) {
+        const int c = threadIdx.x >> 3, j = threadIdx.x & 7;
+        ColSum<T> s = (ColSum<T>(sm.red[j][c]) + ColSum<T>(sm.red[j + 8][c])) + ColSum<T>(sm.red[j + 16][c]);
+#pragma unroll
+        for (int off = 4; off > 0; off >>= 1) s = s + s.shfl(off);
+        if (j == 0) s.store(buf + c * nb + bl);
+    }
+    if (!lane_barrier<ASYNC>(sm, target)) return false;
+    constexpr int CPW = (K + kRunWarps - 1) / kRunWarps, BPL = kRunMaxBlocks / 32;
+    ColSum<T> q[CPW][BPL];
+#pragma unroll
+    for (int i = 0; i < CPW; ++i)
+#pragma unroll
+        for (int b = 0; b < BPL; ++b) {
+            const int c = warp + i * kRunWarps, bb = lane + 32 * b;
+            q[i][b] = c < K && bb < nb ? ColSum<T>::load(buf + c * nb + bb) : ColSum<T>((T)0);
+        }
+#pragma unroll
+    for (int i = 0; i < CPW; ++i) {
+        const int c = warp + i * kRunWarps;
+        ColSum<T> s = ((q[i][0] + q[i][1]) + (q[i][2] + q[i][3])) + q[i][4];
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) s = s + s.shfl(off);
+        if (lane == 0 && c < K) sm.tot[c] = s;
+    }
+    __syncthreads();
+    return true;
+}
+
+// Item `item` of the lane, its tile and rows: the classes of tiles with p up spins in their
+// low part, in falling size, their tiles in order of their high part and each cut into chunks.
+__device__ __forceinline__ void run_item(const uint32_t *sb, const PcgLane &Ln, const uint32_t *cls_item,
+                                         const int *cls_p, int ncls, uint32_t item, uint32_t &t, int &p, uint32_t &jb,
+                                         uint32_t &je)
+{
+    const int B = Ln.B, H = Ln.cp.L - B, m = Ln.cp.n_up;
+    int ci = 0;
+    while (ci + 1 < ncls && item >= cls_item[ci + 1]) ++ci;
+    p = cls_p[ci];
+    const uint32_t Rt = binom(sb, B, p), nch = (Rt + Ln.chunk - 1) / Ln.chunk, rem = item - cls_item[ci];
+    t = cns_unrank(sb, H, m - p, rem / nch);
+    jb = (rem % nch) * Ln.chunk;
+    je = min(Rt, jb + Ln.chunk);
+}
+
+template <typename T>
+__device__ __forceinline__ void run_job(RunShared<T> &sm, uint32_t item, TileJob<T> &job)
+{
+    uint32_t t, jb, je;
+    int p;
+    run_item(sm.binom, sm.lane, sm.cls_item, sm.cls_p, sm.ncls, item, t, p, jb, je);
+    __syncwarp();
+    tile_meta_warp<T>(sm.binom, sm.tab, sm.lane.cp, sm.lane.B, t, p, job.meta);
+    if ((threadIdx.x & 31) == 0) {
+        job.t = t;
+        job.p = p;
+        job.jb = jb;
+        job.je = je;
+    }
+    __syncwarp();
+}
+
+// This worker's share of the items: a warp (or, staged, a group of 256 threads) takes
+// `count` of them, the i-th at item(i).
+struct RunShare {
+    uint32_t first, stride, count;
+    bool there_and_back;
+    __device__ __forceinline__ uint32_t item(uint32_t i) const
+    {
+        return i * stride + ((there_and_back && (i & 1u)) ? stride - 1u - first : first);
+    }
+};
+
+template <bool STAGED>
+__device__ __forceinline__ RunShare run_share(const PcgLane &Ln)
+{
+    const uint32_t nb = Ln.nblocks, bl = blockIdx.x - Ln.block0, warp = threadIdx.x >> 5, items = Ln.items;
+    if (STAGED) {
+        // worker w of W goes through the tiles there and back: w, 2 W - 1 - w, 2 W + w, ...
+        const uint32_t W = nb * kRunSubs, w = bl * kRunSubs + threadIdx.x / kThreads;
+        const uint32_t full = items / W, left = items % W;
+        return RunShare{w, W, full + (left > ((full & 1u) ? W - 1u - w : w) ? 1u : 0u), true};
+    }
+    // the block's even share of the items, dealt out to its warps
+    const uint32_t b0 = (uint32_t)((uint64_t)items * bl / nb), b1 = (uint32_t)((uint64_t)items * (bl + 1) / nb);
+    const uint32_t first = b0 + warp;
+    return RunShare{first, (uint32_t)kRunWarps, first < b1 ? (b1 - first + kRunWarps - 1) / kRunWarps : 0u, false};
+}
+
+// Jobs kept for the whole launch where a worker has few of them (else made each time).
+template <typename T>
+__device__ __forceinline__ void run_cache_jobs(RunShared<T> &sm, const RunShare &sh, bool staged)
+{
+    const uint32_t warp = threadIdx.x >> 5;
+    if (staged) {
+        constexpr uint32_t NJ = kRunJobs / kRunSubs;
+        const uint32_t sub = threadIdx.x / kThreads;
+        if (sh.count <= NJ)
+            for (uint32_t i = warp - sub * kWarps; i < sh.count; i += kWarps)
+                run_job<T>(sm, sh.item(i), sm.jobs[sub * NJ + i]);
+    } else if (sh.count <= 2) {
+        for (uint32_t i = 0; i < sh.count; ++i) run_job<T>(sm, sh.item(i), sm.jobs[2 * warp + i]);
+    }
+}
+
+// The product of this block's jobs: Y = (H - sigma) X and, per column, the warp's sum of
+// y.y (kPcgT), or q = (H - sigma) X, R -= alpha q and the sum of R.(M^-1 R) (kPcgQ), into
+// sm.red.  Staged: a group of 256 threads takes whole tiles, one at a time: the other groups
+// work while its copy is in flight, and a second buffer would come out of the L1 that loads
+// in flight need (L = 20, k = 32: 105 us a step with two buffers, 93 with one).  Else a
+// warp takes a chunk of a tile.
+template <typename T, int K, int MODE, bool STAGED>
+__device__ __noinline__ void run_product()
+{
+    using Lay = WideRowLayout<T, K, run_lane_bytes(K, sizeof(T))>;
+    constexpr int V = Lay::V, G = Lay::G, RPW = 32 / G;
     constexpr int NBr = 128 / (V * (int)sizeof(T));
     constexpr int NB = NBr < 2 ? 2 : (NBr > 8 ? 8 : NBr);
-    __shared__ uint32_t sbin[kBinomDim * kBinomDim];
-    __shared__ T tab[1024];
-    __shared__ T red[kWarps][64];
-    __shared__ uint32_t spref[kLowMaxB + 2];
-    __shared__ T s_alpha[64];
-    __shared__ TileMeta<T> s_meta[kWarps];
-    __shared__ ChainParams s_cp;
-    __shared__ int s_lane;
-    __shared__ unsigned s_last;
-    load_binom(sbin);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, grp = lane / G;
-    const int col = (lane % G) * V;
-    const uint32_t r_begin = (uint32_t)(((uint64_t)total_rounds * blockIdx.x) / gridDim.x);
-    const uint32_t r_end = (uint32_t)(((uint64_t)total_rounds * (blockIdx.x + 1)) / gridDim.x);
-    int cur = -1;
-    for (uint32_t round = r_begin; round < r_end; ++round) {
-        if (threadIdx.x == 0) s_lane = lane_of(lanes, nlanes, round, false);
-        __syncthreads();
-        const int li = s_lane;
-        const PcgLane &Ln = lanes[li];
-        if (li != cur) {
-            // the lane's chain constants, field tables, tile-row prefix and alpha
-            const int *src = reinterpret_cast<const int *>(&Ln.cp);
-            int *dst = reinterpret_cast<int *>(&s_cp);
-            for (int i = threadIdx.x; i < (int)(sizeof(ChainParams) / sizeof(int)); i += kThreads) dst[i] = src[i];
-            __syncthreads();
-            build_field_tables<T>(tab, s_cp);
-            if (MODE == kPcgQ && threadIdx.x < K) s_alpha[threadIdx.x] = (T)Ln.alpha[threadIdx.x];
-            if (threadIdx.x == 0) {
-                const int B = Ln.B;
-                uint32_t acc = 0;
-                for (int q = 0; q <= B + 1 && q <= kLowMaxB + 1; ++q) {
-                    spref[q] = acc;
-                    acc += binom(sbin, B, q);
-                }
-            }
-            __syncthreads();
-            cur = li;
-        }
-        const ChainParams &cp = s_cp;
-        const int B = Ln.B;
-        const int L = cp.L, m = cp.n_up, H = L - B;
-        const uint32_t nchunk = (binom(sbin, B, B / 2) + CH - 1) / CH;
-        const T hdelta = cp_half_delta<T>(cp);
-        T *__restrict__ X = (T *)(MODE == kPcgT ? Ln.p : Ln.t);
-        T *__restrict__ Y = (T *)(MODE == kPcgT ? Ln.t : nullptr);
-        T *__restrict__ R = (T *)(MODE == kPcgQ ? Ln.r : nullptr);
-        const T *__restrict__ dinv = (const T *)Ln.dinv;
-        T part[V];
+    RunShared<T> &sm = run_shared<T>();
+    const PcgLane &Ln = sm.lane;
+    const ChainParams &cp = Ln.cp;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, grp = lane / G, col = (lane % G) * V;
+    const int B = Ln.B, H = cp.L - B;
+    const T hdelta = cp_half_delta<T>(cp);
+    T *X = as_global<T>(MODE == kPcgT ? Ln.p : Ln.t);
+    T *Y = MODE == kPcgT ? as_global<T>(Ln.t) : nullptr;
+    T *R = MODE == kPcgQ ? as_global<T>(Ln.r) : nullptr;
+    const T *dinv = as_global<T>(const_cast<void *>(Ln.dinv));
+    const LowRec *tbl = g_lowtab + lowtab_base(B);
+    const RunShare sh = run_share<STAGED>(Ln);
+    T part[V];
 #pragma unroll
-        for (int v = 0; v < V; ++v) part[v] = (T)0;
-        const uint32_t item = (round - Ln.round0) * kWarps + warp;
-        if (item < Ln.items) {
-            const uint32_t t = item / nchunk, c = item % nchunk;
-            const int p = m - __popc(t);
-            const uint32_t Rt = (p >= 0 && p <= B) ? binom(sbin, B, p) : 0u;
-            const uint32_t j_begin = c * CH;
-            if (j_begin < Rt) {  // warp-uniform
-                const uint32_t j_end = min(Rt, j_begin + CH);
-                TileMeta<T> &tm = s_meta[warp];
-                __syncwarp();
-                tile_meta_warp<T>(sbin, tab, cp, B, t, p, tm);
-                __syncwarp();
-                const uint32_t t0 = t & 1u, thi = (t >> (H - 1)) & 1u;
-                const uint32_t sup = p >= 1 ? binom(sbin, B - 1, p - 1) : 0u;
-                const uint32_t sdn = binom(sbin, B - 1, p);
-                const LowRec *__restrict__ rp = g_lowtab + lowtab_base(B) + spref[p];
-                const T *__restrict__ Xt = X + (int64_t)tm.off * K;
-                for (uint32_t j0 = j_begin; j0 < j_end; j0 += RPW) {
-                    const uint32_t j = j0 + grp;
-                    tile_row_pass<T, V, NB, MODE>(cp, B, X, K, Xt, K, rp, min(j, j_end - 1u), j < j_end, tm, tab,
-                                                  hdelta, t0, thi, sup, sdn, col, Y, K, R, dinv, s_alpha, part,
-                                                  nullptr, nullptr);
-                }
+    for (int v = 0; v < V; ++v) part[v] = (T)0;
+    if (!STAGED) {
+#pragma unroll 1
+        for (uint32_t i = 0; i < sh.count; ++i) {
+            TileJob<T> &job = sm.jobs[2 * warp + (i & 1)];
+            if (sh.count > 2) run_job<T>(sm, sh.item(i), job);
+            const uint32_t jb = job.jb, je = job.je, t = job.t;
+            const int p = job.p;
+            const uint32_t t0 = t & 1u, thi = (t >> (H - 1)) & 1u;
+            const uint32_t sup = p >= 1 ? binom(sm.binom, B - 1, p - 1) : 0u, sdn = binom(sm.binom, B - 1, p);
+            const LowRec *rp = tbl + sm.spref[p];
+            const T *Xt = X + (int64_t)job.meta.off * K;
+#pragma unroll 1
+            for (uint32_t j0 = jb; j0 < je; j0 += RPW) {
+                const uint32_t j = j0 + grp;
+                tile_row_pass<T, V, NB, MODE>(cp, B, X, K, Xt, K, rp, min(j, je - 1u), j < je, job.meta, sm.tab, hdelta,
+                                              t0, thi, sup, sdn, col, Y, K, R, dinv, sm.alpha, part, nullptr, nullptr);
             }
         }
-        // this round's column partials -> the lane's partial slot of the round
+    } else {
+        const int sub = threadIdx.x / kThreads, wsub = warp - sub * kWarps;
+        constexpr int NJ = kRunJobs / kRunSubs, RPB = kWarps * RPW;
+        unsigned char *buf = reinterpret_cast<unsigned char *>(&sm) + run_stage_offset<T>() +
+                             (size_t)sub * Ln.stage_bytes;
+        uint64_t *mbar = &sm.mbar[sub];
+        unsigned parity = sm.parity[warp];
+        auto issue = [&](uint32_t i) {  // by the group's first warp
+            TileJob<T> &job = sm.jobs[sub * NJ + i % NJ];
+            if (sh.count > (uint32_t)NJ) run_job<T>(sm, sh.item(i), job);
+            if (lane == 0) {
+                const unsigned bytes = job.je * (unsigned)(K * sizeof(T));
+                fence_proxy_async();
+                mbar_arrive_expect_tx(mbar, bytes);
+                bulk_copy_g2s(buf, X + (int64_t)job.meta.off * K, bytes, mbar);
+            }
+        };
+        if (wsub == 0 && sh.count > 0) issue(0);
+#pragma unroll 1
+        for (uint32_t i = 0; i < sh.count; ++i) {
+            if (!mbar_wait_bounded(mbar, parity)) {
+                // wait once more so that no copy is left in flight, and fail the lane
+                mbar_wait_bounded(mbar, parity);
+                atomicExch(Ln.counter + 3, 1u);
+            }
+            parity ^= 1u;
+            const TileJob<T> &job = sm.jobs[sub * NJ + i % NJ];
+            const uint32_t je = job.je, t = job.t;
+            const int p = job.p;
+            const uint32_t t0 = t & 1u, thi = (t >> (H - 1)) & 1u;
+            const uint32_t sup = p >= 1 ? binom(sm.binom, B - 1, p - 1) : 0u, sdn = binom(sm.binom, B - 1, p);
+            const LowRec *rp = tbl + sm.spref[p];
+            const T *Xt = reinterpret_cast<const T *>(buf);
+#pragma unroll 1
+            for (uint32_t j0 = wsub * RPW; j0 < je; j0 += RPB) {
+                const uint32_t j = j0 + grp;
+                tile_row_pass<T, V, NB, MODE>(cp, B, X, K, Xt, K, rp, min(j, je - 1u), j < je, job.meta, sm.tab,
+                                              hdelta, t0, thi, sup, sdn, col, Y, K, R, dinv, sm.alpha, part,
+                                              nullptr, nullptr);
+            }
+            // every read of this buffer and job is done before they are filled again
+            asm volatile("bar.sync %0, %1;" ::"r"(1 + sub), "r"(kThreads) : "memory");
+            if (wsub == 0 && i + 1 < sh.count) issue(i + 1);
+        }
+        if (lane == 0) sm.parity[warp] = parity;
+    }
 #pragma unroll
-        for (int v = 0; v < V; ++v)
-            for (int off = G; off < 32; off <<= 1) part[v] += __shfl_xor_sync(0xffffffffu, part[v], off);
-        if (lane < G) {
+    for (int v = 0; v < V; ++v)
+        for (int off = G; off < 32; off <<= 1) part[v] += __shfl_xor_sync(0xffffffffu, part[v], off);
+    if (lane < G) {
 #pragma unroll
-            for (int v = 0; v < V; ++v) red[warp][lane * V + v] = part[v];
-        }
-        __syncthreads();
-        const uint32_t slot = round - Ln.round0;
-        if (threadIdx.x < K) {
-            if constexpr (sizeof(T) == 4) {
-                float sum = 0.0f, cmp = 0.0f;
-                for (int w = 0; w < kWarps; ++w) {
-                    float hi, e;
-                    two_sum(sum, red[w][threadIdx.x], hi, e);
-                    sum = hi;
-                    cmp += e;
-                }
-                reinterpret_cast<float2 *>(Ln.partials)[(int64_t)slot * K + threadIdx.x] = make_float2(sum, cmp);
-            } else {
-                double acc = 0.0;
-                for (int w = 0; w < kWarps; ++w) acc += (double)red[w][threadIdx.x];
-                Ln.partials[(int64_t)slot * K + threadIdx.x] = acc;
-            }
-        }
-        __threadfence();
-        __syncthreads();
-        if (threadIdx.x == 0) s_last = (atomicAdd(Ln.counter, 1u) == Ln.nrounds - 1) ? 1u : 0u;
-        __syncthreads();
-        if (s_last) {
-            // this block finished the lane's last round: sum the rounds in order
-            __threadfence();
-            if (threadIdx.x < K) {
-                double tot;
-                if constexpr (sizeof(T) == 4) {
-                    const float2 *pp = reinterpret_cast<const float2 *>(Ln.partials);
-                    float S = 0.0f, C = 0.0f;
-                    for (uint32_t q = 0; q < Ln.nrounds; ++q) {
-                        const float2 v2 = pp[(int64_t)q * K + threadIdx.x];
-                        float hi, e;
-                        two_sum(S, v2.x, hi, e);
-                        S = hi;
-                        C += e + v2.y;
-                    }
-                    tot = (double)S + (double)C;
-                } else {
-                    double S = 0.0;
-                    for (uint32_t q = 0; q < Ln.nrounds; ++q) S += Ln.partials[(int64_t)q * K + threadIdx.x];
-                    tot = S;
-                }
-                const int cc = threadIdx.x;
-                if (MODE == kPcgT) {
-                    const bool ok = Ln.active[cc] && tot > 0.0 && isfinite(tot);
-                    Ln.alpha[cc] = ok ? Ln.rz[cc] / tot : 0.0;
-                } else {
-                    int act = Ln.active[cc];
-                    if (!isfinite(tot)) act = 0;
-                    if (Ln.tol2 > 0.0 && tot <= Ln.tol2 * Ln.rz0[cc]) act = 0;
-                    Ln.beta[cc] = (act && Ln.rz[cc] > 0.0) ? tot / Ln.rz[cc] : 0.0;
-                    if (!act) Ln.alpha[cc] = 0.0;
-                    Ln.active[cc] = act;
-                    Ln.rz[cc] = tot;
-                }
-            }
-            if (threadIdx.x == 0) *Ln.counter = 0u;
-        }
+        for (int v = 0; v < V; ++v) sm.red[warp][lane * V + v] = part[v];
     }
 }
 
-// Batched direction update: w += alpha p, p = M^-1 r + beta p for every lane's rows (the
-// lanes' rows concatenated; each thread takes kUpdRows rows, loads first).
-template <typename T, int K>
-__global__ void __launch_bounds__(kThreads) k_pcg_batch_update(const PcgLane *__restrict__ lanes, int nlanes,
-                                                               uint32_t total_rows)
+// Tensor memory as storage that a thread alone uses: its lane of the SM's 128, its warp's
+// 84 of the 512 columns, four 32-bit words a slot.
+__device__ __forceinline__ uint32_t run_tmem_slot(uint32_t base, uint32_t slot)
 {
-    using Lay = RowLayout<T, K>;
-    constexpr int V = Lay::V, G = Lay::G;
-    const int col = (threadIdx.x % G) * V;
-    const uint32_t rows_per_block = kThreads / G;
-    const uint64_t stride = (uint64_t)gridDim.x * rows_per_block * kUpdRows;
-    for (uint64_t base = (uint64_t)blockIdx.x * rows_per_block * kUpdRows + threadIdx.x / G; base < total_rows;
-         base += stride) {
-        Vec<T, V> rv[kUpdRows], pv[kUpdRows], wv[kUpdRows];
-        T di[kUpdRows];
-        int li[kUpdRows];
-        int64_t o[kUpdRows];
-#pragma unroll
-        for (int q = 0; q < kUpdRows; ++q) {
-            uint64_t row = base + (uint64_t)q * rows_per_block;
-            if (row >= total_rows) row = total_rows - 1;  // a valid row; stored only if in range
-            li[q] = lane_of(lanes, nlanes, (uint32_t)row, true);
-            const PcgLane &Ln = lanes[li[q]];
-            const uint32_t lr = (uint32_t)row - Ln.row0;
-            o[q] = (int64_t)lr * K + col;
-            rv[q] = ldv<T, V>((const T *)Ln.r + o[q]);
-            pv[q] = ldv<T, V>((const T *)Ln.p + o[q]);
-            wv[q] = ldv<T, V>((const T *)Ln.w + o[q]);
-            di[q] = ((const T *)Ln.dinv)[lr];
+    const uint32_t warp = threadIdx.x >> 5;
+    return base + ((warp & 3u) << 21) + (warp >> 2) * (4u * kRunSlots) + 4u * slot;
+}
+
+__device__ __forceinline__ uint4 tmem_ld4(uint32_t addr)
+{
+    uint4 v;
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%4];\n\t"
+                 "tcgen05.wait::ld.sync.aligned;"
+                 : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
+                 : "r"(addr)
+                 : "memory");
+    return v;
+}
+
+__device__ __forceinline__ void tmem_st4(uint32_t addr, const uint4 &v)
+{
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(v.x), "r"(v.y),
+                 "r"(v.z), "r"(v.w)
+                 : "memory");
+}
+
+__device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
+
+// Rows of the block's share: slot s of thread x is row row_b + s * RPP + x / G.
+template <typename T, int K>
+struct RunRows {
+    static constexpr int V = RowLayout<T, K>::V, G = RowLayout<T, K>::G, RPP = kRunThreads / G;
+    static_assert(V * sizeof(T) == 16, "four 32-bit words a slot");
+};
+
+// The block's rows of w into tensor memory (LOAD), or back.
+template <typename T, int K, bool LOAD>
+__device__ __forceinline__ void run_move_w(uint32_t row_b, uint32_t row_e, uint32_t tmem)
+{
+    using Rows = RunRows<T, K>;
+    T *w = as_global<T>(run_shared<T>().lane.w);
+    const uint32_t slots = (row_e - row_b + Rows::RPP - 1) / Rows::RPP;
+#pragma unroll 1
+    for (uint32_t s = 0; s < slots; ++s) {  // the same for all threads: tcgen05 wants whole warps
+        const uint32_t row = row_b + s * Rows::RPP + threadIdx.x / Rows::G;
+        uint4 *g = reinterpret_cast<uint4 *>(w + (int64_t)row * K + (threadIdx.x % Rows::G) * Rows::V);
+        if (LOAD) {
+            tmem_st4(run_tmem_slot(tmem, s), row < row_e ? *g : make_uint4(0, 0, 0, 0));
+        } else {
+            const uint4 v = tmem_ld4(run_tmem_slot(tmem, s));
+            if (row < row_e) *g = v;
         }
+    }
+    if (LOAD) tmem_wait_st();
+}
+
+// w += alpha p, p = M^-1 r + beta p for rows [row_b, row_e), the block's share.  W_TMEM: w
+// stays in tensor memory for the whole launch, which takes two of the phase's five vector
+// streams off L2 (L = 20, k = 32: 25 -> 18 us for this phase; then three rows a thread in
+// flight instead of five, which spilled, 18 -> 13 us).
+constexpr int kRunUpdRows = 3;
+template <typename T, int K, bool W_TMEM>
+__device__ __noinline__ void run_update(uint32_t row_b, uint32_t row_e, uint32_t tmem)
+{
+    using Rows = RunRows<T, K>;
+    constexpr int V = Rows::V, G = Rows::G, RPP = Rows::RPP, U = kRunUpdRows;
+    RunShared<T> &sm = run_shared<T>();
+    const int col = (threadIdx.x % G) * V;
+    T a[V], bt[V];
 #pragma unroll
-        for (int q = 0; q < kUpdRows; ++q) {
-            if (base + (uint64_t)q * rows_per_block >= total_rows) continue;
-            const PcgLane &Ln = lanes[li[q]];
-            Vec<T, V> pn;
+    for (int v = 0; v < V; ++v) {
+        a[v] = sm.alpha[col + v];
+        bt[v] = sm.beta[col + v];
+    }
+    const uint32_t slots = (row_e - row_b + RPP - 1) / RPP;
+    uint32_t row = row_b + threadIdx.x / G;
+    // the thread's rows lie RPP apart: constant offsets from these pointers
+    const int64_t at0 = (int64_t)row * K + col;
+    const T *r = as_global<T>(sm.lane.r) + at0, *dinv = as_global<T>(const_cast<void *>(sm.lane.dinv)) + row;
+    T *p = as_global<T>(sm.lane.p) + at0, *w = as_global<T>(sm.lane.w) + at0;
+    constexpr int STEP = RPP * K;
+    uint32_t slot = W_TMEM ? run_tmem_slot(tmem, 0) : 0u;
+#pragma unroll 1
+    for (uint32_t s0 = 0; s0 < slots; s0 += U) {
+        Vec<T, V> rv[U], pv[U];
+        T di[U];
 #pragma unroll
-            for (int v = 0; v < V; ++v) {
-                const T a = (T)Ln.alpha[col + v], bt = (T)Ln.beta[col + v];
-                wv[q].v[v] += a * pv[q].v[v];
-                pn.v[v] = di[q] * rv[q].v[v] + bt * pv[q].v[v];
+        for (int q = 0; q < U; ++q)
+            if (row + q * RPP < row_e) {
+                rv[q] = ldv<T, V>(r + q * STEP);
+                pv[q] = ldv<T, V>(p + q * STEP);
+                di[q] = dinv[q * RPP];
             }
-            stv<T, V>((T *)Ln.w + o[q], wv[q]);
-            stv<T, V>((T *)Ln.p + o[q], pn);
+#pragma unroll
+        for (int q = 0; q < U; ++q) {
+            if (s0 + q >= slots) break;
+            const bool in = row + q * RPP < row_e;
+            if (W_TMEM) {
+                uint4 raw = tmem_ld4(slot + 4 * q);
+                Vec<T, V> wv = *reinterpret_cast<Vec<T, V> *>(&raw);
+#pragma unroll
+                for (int v = 0; v < V; ++v) wv.v[v] += a[v] * (in ? pv[q].v[v] : (T)0);
+                tmem_st4(slot + 4 * q, *reinterpret_cast<uint4 *>(&wv));
+            } else if (in) {
+                Vec<T, V> wv = ldv<T, V>(w + q * STEP);
+#pragma unroll
+                for (int v = 0; v < V; ++v) wv.v[v] += a[v] * pv[q].v[v];
+                stv<T, V>(w + q * STEP, wv);
+            }
+            if (in) {
+                Vec<T, V> pn;
+#pragma unroll
+                for (int v = 0; v < V; ++v) pn.v[v] = di[q] * rv[q].v[v] + bt[v] * pv[q].v[v];
+                stv<T, V>(p + q * STEP, pn);
+            }
+        }
+        row += U * RPP;
+        r += U * STEP;
+        p += U * STEP;
+        w += U * STEP;
+        dinv += U * RPP;
+        slot += 4 * U;
+    }
+    if (W_TMEM) tmem_wait_st();
+}
+
+template <typename T, int K, bool STAGED>
+__global__ void __launch_bounds__(kRunThreads, 1)
+    k_pcg_run(const __grid_constant__ PcgLane one, const PcgLane *lanes, int nlanes, int steps)
+{
+    RunShared<T> &sm = run_shared<T>();
+    const PcgLane &Ln = sm.lane;
+    {
+        // the lane this block serves
+        const PcgLane *src = &one;
+        if (lanes) {
+            int lo = 0, hi = nlanes - 1;
+            while (lo < hi) {
+                const int mid = (lo + hi + 1) >> 1;
+                if (lanes[mid].block0 <= blockIdx.x) lo = mid;
+                else hi = mid - 1;
+            }
+            src = lanes + lo;
+        }
+        const int *s = reinterpret_cast<const int *>(src);
+        int *d = reinterpret_cast<int *>(&sm.lane);
+        for (int i = threadIdx.x; i < (int)(sizeof(PcgLane) / sizeof(int)); i += kRunThreads) d[i] = s[i];
+    }
+    load_binom(sm.binom);
+    if (STAGED && threadIdx.x < kRunSubs) mbar_init(&sm.mbar[threadIdx.x], 1);
+    if (threadIdx.x < kRunWarps) sm.parity[threadIdx.x] = 0;
+    __syncthreads();
+    build_field_tables<T>(sm.tab, Ln.cp);
+    if (threadIdx.x == 0) {
+        const int B = Ln.B;
+        uint32_t acc = 0;
+        for (int q = 0; q <= B + 1 && q <= kLowMaxB + 1; ++q) {
+            sm.spref[q] = acc;
+            acc += binom(sm.binom, B, q);
+        }
+    }
+    if (threadIdx.x == 32) {  // the classes of tiles in falling size
+        const int B = Ln.B, H = Ln.cp.L - B, m = Ln.cp.n_up;
+        int n = 0;
+        for (int p = max(0, m - H); p <= min(B, m); ++p) {
+            int i = n++;
+            for (; i > 0 && binom(sm.binom, B, sm.cls_p[i - 1]) < binom(sm.binom, B, p); --i)
+                sm.cls_p[i] = sm.cls_p[i - 1];
+            sm.cls_p[i] = p;
+        }
+        uint32_t acc = 0;
+        for (int i = 0; i < n; ++i) {
+            const int p = sm.cls_p[i];
+            sm.cls_item[i] = acc;
+            acc += binom(sm.binom, H, m - p) * ((binom(sm.binom, B, p) + Ln.chunk - 1) / Ln.chunk);
+        }
+        sm.ncls = n;
+    }
+    if (threadIdx.x >= 64 && threadIdx.x < 64 + K) {
+        const int c = threadIdx.x - 64;
+        sm.rz[c] = ColSum<T>::of(Ln.rz[c]);
+        sm.active[c] = Ln.active[c];
+    }
+    __syncthreads();
+    const uint32_t nb = Ln.nblocks, bl = blockIdx.x - Ln.block0;
+    const uint32_t row_b = (uint32_t)((uint64_t)Ln.n * bl / nb), row_e = (uint32_t)((uint64_t)Ln.n * (bl + 1) / nb);
+    // w in tensor memory when the block's rows fit there
+    const bool w_tmem = row_e - row_b <= (uint32_t)(kRunSlots * RunRows<T, K>::RPP);
+    if (w_tmem && threadIdx.x < 32) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_addr(&sm.tmem)),
+                     "r"(512)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    run_cache_jobs<T>(sm, run_share<STAGED>(Ln), STAGED);
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    const uint32_t tmem = w_tmem ? sm.tmem : 0u;
+    if (w_tmem) run_move_w<T, K, true>(row_b, row_e, tmem);
+    unsigned target = 0;
+    bool ok = true;
+#pragma unroll 1
+    for (int step = 0; step < steps; ++step) {
+        run_product<T, K, kPcgT, STAGED>();
+        if (!(ok = lane_column_sums<T, K, STAGED>(Ln.partials, target))) break;
+        if (threadIdx.x < K) {
+            const int c = threadIdx.x;
+            const ColSum<T> tt = sm.tot[c];
+            sm.alpha[c] = sm.active[c] && tt.positive() ? sm.rz[c].over(tt) : (T)0;
+        }
+        __syncthreads();
+        run_product<T, K, kPcgQ, STAGED>();
+        if (!(ok = lane_column_sums<T, K, STAGED>(Ln.partials + (size_t)nb * K, target))) break;
+        if (threadIdx.x < K) {
+            // beta, and the freeze rule: a column stops once rz <= tol^2 rz0, or on NaN/Inf
+            const int c = threadIdx.x;
+            const ColSum<T> rzn = sm.tot[c], rz = sm.rz[c];
+            int act = sm.active[c] && rzn.finite();
+            if (Ln.tol2 > 0.0 && rzn.value() <= Ln.tol2 * Ln.rz0[c]) act = 0;
+            const T b = act && rz.positive() ? rzn.over(rz) : (T)0;
+            sm.beta[c] = b;
+            if (!act) sm.alpha[c] = (T)0;
+            sm.active[c] = act;
+            sm.rz[c] = rzn;
+            if (bl == 0 && step == steps - 1) {
+                Ln.rz[c] = rzn.value();
+                Ln.alpha[c] = (double)sm.alpha[c];
+                Ln.beta[c] = (double)b;
+                Ln.active[c] = act;
+            }
+        }
+        __syncthreads();
+        if (w_tmem) run_update<T, K, true>(row_b, row_e, tmem);
+        else run_update<T, K, false>(row_b, row_e, 0u);
+        if (step + 1 < steps && !(ok = lane_barrier<STAGED>(sm, target))) break;
+    }
+    if (w_tmem && ok) run_move_w<T, K, false>(row_b, row_e, tmem);
+    if (!ok && row_b < row_e && threadIdx.x < K)
+        static_cast<T *>(Ln.w)[(int64_t)row_b * K + threadIdx.x] = (T)NAN;
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    if (w_tmem && threadIdx.x < 32)
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512) : "memory");
+    // the last block to leave puts the barrier words back to zero
+    if (nb > 1 && threadIdx.x == 0) {
+        __threadfence();
+        if (atomicAdd(Ln.counter + 2, 1u) == nb - 1u) {
+            Ln.counter[1] = 0u;
+            Ln.counter[2] = 0u;
         }
     }
 }
@@ -2908,84 +3346,175 @@ template int pcg_start<float>(const double *, int64_t, const double *, uint32_t,
 template int pcg_start<double>(const double *, int64_t, const double *, uint32_t, int, const double *, double *,
                                double *, double *, const PcgDev &, cudaStream_t);
 
-// ---- batched PCG step: host side ------------------------------------------------
+// ---- resident PCG: host side -----------------------------------------------------
 
-// Work items and rounds of one lane (the persistent tiled product's items: a chunk of
-// WideRowLayout::CH rows of one tile, all 2^(L-B) tiles).
-template <typename T, int K>
-static void lane_items(int L, int B, uint32_t *items, uint32_t *nrounds)
+constexpr double kRunL2Bytes = 100e6;
+// Row passes a block gets at least: fewer warps on more SMs share out the L2 latency and
+// bandwidth of a small problem (L = 16, k = 16: 23 us a step with 24 passes a block, 17.9
+// with 12, 17.3 with 6, 16.9 with 3), against a barrier among more blocks.
+constexpr uint64_t kRunSpread = 3;
+
+// Rows that one pass of a warp covers.
+static uint32_t run_rows_per_pass(int K, size_t es)
 {
-    constexpr int CH = WideRowLayout<T, K, 32>::CH;
-    const uint32_t nchunk = (host_binom(B, B / 2) + CH - 1) / CH;
-    *items = (uint32_t)(((uint64_t)1 << (L - B)) * nchunk);
-    *nrounds = (*items + kWarps - 1) / kWarps;
+    const int row = K * (int)es, lb = run_lane_bytes(K, es);
+    return 32u / (uint32_t)(row >= lb ? row / lb : 1);
+}
+
+// How the products of a lane are split, from its sizes alone.
+static bool run_staged(int L, int n_up, int K, size_t es)
+{
+    return (K * (int)es) % 16 == 0 && schedule_for(L, n_up, K, es) == 3;
+}
+
+static int run_staged_bits(int L, int K, size_t es)
+{
+    int B = kLowMaxB < L - 2 ? kLowMaxB : L - 2;
+    while (B >= 2 && (size_t)host_binom(B, B / 2) * K * es > (size_t)kRunStageBytes) --B;
+    return B;
+}
+
+// Row passes of all tiles, and work items for a chunk of `chunk` rows.
+static uint64_t run_items(int L, int n_up, int B, uint32_t chunk)
+{
+    uint64_t items = 0;
+    const int H = L - B;
+    for (int p = 0; p <= B; ++p)
+        if (n_up - p >= 0 && n_up - p <= H)
+            items += (uint64_t)host_binom(H, n_up - p) * ((host_binom(B, p) + chunk - 1) / chunk);
+    return items;
+}
+
+uint64_t pcg_lane_passes(int L, int n_up, int k, int f32)
+{
+    const size_t es = f32 ? 4 : 8;
+    const int B = tile_bits_for(L, k, es);
+    return B < 2 ? 0 : run_items(L, n_up, B, run_rows_per_pass(k, es));
+}
+
+// The resident kernel serves the tiled widths under the default switches, while a lane's
+// four vectors stay in L2; a work order or lane width asked for explicitly
+// (mbl_set_product_schedule 4 and 5, mbl_set_product_lane_bytes) keeps its own launches.
+bool pcg_run_supported(int L, int n_up, int k, int f32)
+{
+    const size_t es = f32 ? 4 : 8;
+    if ((double)host_binom(L, n_up) * k * (double)es * 4.0 > kRunL2Bytes) return false;
+    if (k != 8 && k != 16 && k != 32 && k != 64) return false;
+    if (tile_bits_for(L, k, es) < 2) return false;
+    const int o = g_schedule[es == 8 ? 1 : 0][kslot(k)], lb = g_lane_bytes[es == 8 ? 1 : 0][kslot(k)];
+    return o != 4 && o != 5 && lb == 0;
 }
 
 int pcg_lane_fill(PcgLane *Ln, const ChainParams &cp, uint32_t n, int k, int f32, const void *dinv, void *r,
-                  void *p, void *t, void *w, const PcgDev &pd, uint32_t *round0, uint32_t *row0)
+                  void *p, void *t, void *w, const PcgDev &pd, uint32_t block0, uint32_t max_blocks, bool may_stage)
 {
     const size_t es = f32 ? 4 : 8;
-    const int B = tile_bits_for(cp.L, k, es);
-    if (B < 2) return MBL_ERR_ARG;
-    if (ensure_lowtab(B) != MBL_OK) return MBL_ERR_CUDA;
-    uint32_t items = 0, nrounds = 0;
-    switch (k) {
-    case 8: f32 ? lane_items<float, 8>(cp.L, B, &items, &nrounds) : lane_items<double, 8>(cp.L, B, &items, &nrounds); break;
-    case 16: f32 ? lane_items<float, 16>(cp.L, B, &items, &nrounds) : lane_items<double, 16>(cp.L, B, &items, &nrounds); break;
-    case 32: f32 ? lane_items<float, 32>(cp.L, B, &items, &nrounds) : lane_items<double, 32>(cp.L, B, &items, &nrounds); break;
-    case 64: f32 ? lane_items<float, 64>(cp.L, B, &items, &nrounds) : lane_items<double, 64>(cp.L, B, &items, &nrounds); break;
-    default: return MBL_ERR_ARG;
+    if (!pcg_run_supported(cp.L, cp.n_up, k, f32) || max_blocks < 1) return MBL_ERR_ARG;
+    const uint32_t rpw = run_rows_per_pass(k, es);
+    PcgLane o{};
+    o.cp = cp;
+    o.dinv = dinv;
+    o.r = r;
+    o.p = p;
+    o.t = t;
+    o.w = w;
+    o.rz = pd.rz;
+    o.rz0 = pd.rz0;
+    o.alpha = pd.alpha;
+    o.beta = pd.beta;
+    o.active = pd.active;
+    o.tol2 = pd.tol2;
+    o.partials = pd.partials;
+    o.counter = pd.counter;
+    o.n = n;
+    o.block0 = block0;
+    if (max_blocks > (uint32_t)kRunMaxBlocks) max_blocks = kRunMaxBlocks;
+    const int Bs = may_stage && run_staged(cp.L, cp.n_up, k, es) ? run_staged_bits(cp.L, k, es) : -1;
+    if (Bs >= 2) {
+        o.B = Bs;
+        o.chunk = host_binom(o.B, o.B / 2);
+        o.stage_bytes = o.chunk * (uint32_t)(k * es);
+        o.nblocks = max_blocks;
+    } else {
+        o.B = tile_bits_for(cp.L, k, es);
+        const uint64_t passes = run_items(cp.L, cp.n_up, o.B, rpw);
+        const uint64_t need = (passes + kRunSpread - 1) / kRunSpread;
+        o.nblocks = (uint32_t)(need < max_blocks ? need : max_blocks);
+        const uint64_t warps = (uint64_t)o.nblocks * kRunWarps;
+        uint32_t best = 1;
+        double best_cost = 0.0;
+        // passes per item: the fewest rounds of passes, an item's set-up counted as half a pass
+        for (uint32_t q = 1; q <= 16; ++q) {
+            const uint64_t items = run_items(cp.L, cp.n_up, o.B, rpw * q);
+            const double cost = (double)((items + warps - 1) / warps) * (q + 0.5);
+            if (q == 1 || cost < best_cost) {
+                best = q;
+                best_cost = cost;
+            }
+        }
+        o.chunk = rpw * best;
     }
-    // the lane's round partials live in its PCG partials buffer
-    if ((size_t)nrounds * k > pcg_partial_doubles()) return MBL_ERR_ARG;
-    *Ln = PcgLane{cp, dinv, r, p, t, w, pd.rz, pd.rz0, pd.alpha, pd.beta, pd.active, pd.tol2, pd.partials,
-                  pd.counter, n, B, items, *round0, nrounds, *row0};
-    *round0 += nrounds;
-    *row0 += n;
+    if (ensure_lowtab(o.B) != MBL_OK) return MBL_ERR_CUDA;
+    o.items = (uint32_t)run_items(cp.L, cp.n_up, o.B, o.chunk);
+    *Ln = o;
     return MBL_OK;
 }
 
-template <typename T, int K>
-static cudaError_t pcg_batch_step_k(const PcgLane *lanes, int nlanes, uint32_t rounds, uint32_t rows, cudaStream_t st)
+template <typename T, int K, bool STAGED>
+static cudaError_t pcg_run_launch(const PcgLane *one, const PcgLane *lanes_dev, int nlanes, uint32_t blocks,
+                                  size_t dyn, int steps, cudaStream_t st)
 {
-    static const int per_sm = [&]() {
-        int v = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, k_pcg_batch<T, K, kPcgT, 32>, kThreads, 0) != cudaSuccess ||
-            v < 1)
-            v = 1;
-        return v;
-    }();
-    int64_t grid = (int64_t)num_sms() * per_sm;
-    if (grid > rounds) grid = rounds;
+    auto kern = k_pcg_run<T, K, STAGED>;
+    constexpr size_t state = run_stage_offset<T>();
+    static const cudaError_t attr = cudaFuncSetAttribute(
+        kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(state + (STAGED ? kRunSubs * kRunStageBytes : 0)));
+    if (attr != cudaSuccess) return attr;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(blocks);
+    cfg.blockDim = dim3(kRunThreads);
+    cfg.dynamicSmemBytes = state + dyn;
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeCooperative;
+    at[0].val.cooperative = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
     note_launch();
-    k_pcg_batch<T, K, kPcgT, 32><<<(int)grid, kThreads, 0, st>>>(lanes, nlanes, rounds);
-    note_launch();
-    k_pcg_batch<T, K, kPcgQ, 32><<<(int)grid, kThreads, 0, st>>>(lanes, nlanes, rounds);
-    int ugrid = (int)(((int64_t)rows * RowLayout<T, K>::G + kThreads * kUpdRows - 1) / (kThreads * kUpdRows));
-    if (ugrid > num_sms() * 8) ugrid = num_sms() * 8;
-    if (ugrid < 1) ugrid = 1;
-    note_launch();
-    k_pcg_batch_update<T, K><<<ugrid, kThreads, 0, st>>>(lanes, nlanes, rows);
-    return cudaGetLastError();
+    return cudaLaunchKernelEx(&cfg, kern, one ? *one : PcgLane{}, lanes_dev, nlanes, steps);
 }
 
-int pcg_batch_step(int f32, const PcgLane *lanes_dev, int nlanes, int k, uint32_t rounds, uint32_t rows,
-                   cudaStream_t st)
+template <typename T, int K>
+static cudaError_t pcg_run_k(const PcgLane *one, const PcgLane *lanes_dev, int nlanes, uint32_t blocks,
+                             uint32_t stage_bytes, int steps, cudaStream_t st)
 {
-    if (nlanes < 1 || rounds < 1 || rows < 1) return MBL_ERR_ARG;
-    cudaError_t e;
-    switch (k) {
-    case 8: e = f32 ? pcg_batch_step_k<float, 8>(lanes_dev, nlanes, rounds, rows, st)
-                    : pcg_batch_step_k<double, 8>(lanes_dev, nlanes, rounds, rows, st); break;
-    case 16: e = f32 ? pcg_batch_step_k<float, 16>(lanes_dev, nlanes, rounds, rows, st)
-                     : pcg_batch_step_k<double, 16>(lanes_dev, nlanes, rounds, rows, st); break;
-    case 32: e = f32 ? pcg_batch_step_k<float, 32>(lanes_dev, nlanes, rounds, rows, st)
-                     : pcg_batch_step_k<double, 32>(lanes_dev, nlanes, rounds, rows, st); break;
-    case 64: e = f32 ? pcg_batch_step_k<float, 64>(lanes_dev, nlanes, rounds, rows, st)
-                     : pcg_batch_step_k<double, 64>(lanes_dev, nlanes, rounds, rows, st); break;
-    default: return MBL_ERR_ARG;
+    if (stage_bytes)
+        return pcg_run_launch<T, K, true>(one, lanes_dev, nlanes, blocks, (size_t)stage_bytes * kRunSubs, steps, st);
+    return pcg_run_launch<T, K, false>(one, lanes_dev, nlanes, blocks, 0, steps, st);
+}
+
+int pcg_run(int f32, const PcgLane *one, const PcgLane *lanes_dev, int nlanes, int k, uint32_t blocks,
+            uint32_t stage_bytes, int steps, cudaStream_t st)
+{
+    if (nlanes < 1 || blocks < 1 || (int)blocks > num_sms() || steps < 0) return MBL_ERR_ARG;
+    // a launch holds the GPU until its last step: at most kRunSteps steps each
+    constexpr int kRunSteps = 64;
+    for (int done = 0; done < steps; done += kRunSteps) {
+        const int now = steps - done < kRunSteps ? steps - done : kRunSteps;
+        cudaError_t e;
+        switch (k) {
+        case 8: e = f32 ? pcg_run_k<float, 8>(one, lanes_dev, nlanes, blocks, stage_bytes, now, st)
+                        : pcg_run_k<double, 8>(one, lanes_dev, nlanes, blocks, stage_bytes, now, st); break;
+        case 16: e = f32 ? pcg_run_k<float, 16>(one, lanes_dev, nlanes, blocks, stage_bytes, now, st)
+                         : pcg_run_k<double, 16>(one, lanes_dev, nlanes, blocks, stage_bytes, now, st); break;
+        case 32: e = f32 ? pcg_run_k<float, 32>(one, lanes_dev, nlanes, blocks, stage_bytes, now, st)
+                         : pcg_run_k<double, 32>(one, lanes_dev, nlanes, blocks, stage_bytes, now, st); break;
+        case 64: e = f32 ? pcg_run_k<float, 64>(one, lanes_dev, nlanes, blocks, stage_bytes, now, st)
+                         : pcg_run_k<double, 64>(one, lanes_dev, nlanes, blocks, stage_bytes, now, st); break;
+        default: return MBL_ERR_ARG;
+        }
+        if (e != cudaSuccess) return MBL_ERR_CUDA;
     }
-    return e == cudaSuccess ? MBL_OK : MBL_ERR_CUDA;
+    return MBL_OK;
 }
 
 template <typename T, int K>
@@ -3019,7 +3548,7 @@ static cudaError_t pcg_step_k(const ChainParams &cp, uint32_t n, const T *dinv, 
     return cudaGetLastError();
 }
 
-// One PCG iteration on A = (H - sigma)^2: t = (H - sigma)p, alpha; r -= alpha (H - sigma)t,
+// One PCG iteration of the widths and switches without a resident kernel, on A = (H - sigma)^2: t = (H - sigma)p, alpha; r -= alpha (H - sigma)t,
 // beta; w += alpha p, p = M^-1 r + beta p.  Three launches, no host synchronisation.
 template <typename T>
 int pcg_step(const ChainParams &cp, uint32_t n, int k, const T *dinv, T *r, T *p, T *t, T *w, const PcgDev &pd,

@@ -106,8 +106,8 @@ struct ChainParams {
     float half_delta_f, diag_const_f;  // rounded once
 };
 
-// One problem (lane) of a batched PCG launch: its chain, vectors, per-column scalars and
-// its place in the launch's rounds and concatenated rows (filled by pcg_lane_fill).
+// One problem (lane) of a resident PCG launch: its chain, vectors, per-column scalars, and
+// the blocks and the split of the products that it was given (filled by pcg_lane_fill).
 struct PcgLane {
     ChainParams cp;
     const void *dinv;
@@ -115,14 +115,14 @@ struct PcgLane {
     double *rz, *rz0, *alpha, *beta;
     int *active;
     double tol2;
-    double *partials;   // >= nrounds * 64 doubles
-    unsigned *counter;  // zero between launches (the finishing block resets it)
+    double *partials;   // >= 2 * nblocks * k doubles
+    unsigned *counter;  // [1] barrier, [2] exit tickets (both zero between launches), [3] fail
     uint32_t n;
     int B;              // tile width
-    uint32_t items;     // work items of the lane
-    uint32_t round0;    // first round of the lane
-    uint32_t nrounds;   // ceil(items / kWarps)
-    uint32_t row0;      // first row of the lane in the concatenated rows (update launch)
+    uint32_t block0, nblocks;  // blocks block0 .. block0 + nblocks - 1 serve this lane
+    uint32_t items;     // units of product work: chunks of tiles, or whole tiles when staged
+    uint32_t chunk;     // rows of an item, at most
+    uint32_t stage_bytes;  // staged: the largest tile's bytes, else 0
 };
 
 // The chain constants in the kernel's own type.

@@ -55,14 +55,19 @@ int pcg_start(const double *B, int64_t ldb, const double *bnorm, uint32_t n, int
 template <typename T>
 int pcg_step(const ChainParams &cp, uint32_t n, int k, const T *dinv, T *r, T *p, T *t, T *w, const PcgDev &pd,
              cudaStream_t st);
-// Batched PCG step over nlanes problems (lanes_dev: a device copy of PcgLane entries filled
-// by pcg_lane_fill, in round order); every lane has block width k, FP32 (f32) or FP64
-// vectors.  Three launches for all lanes.
+// Resident PCG: `steps` PCG steps of one problem (`one`, lanes_dev null) or of nlanes
+// problems (lanes_dev: a device copy of PcgLane entries filled by pcg_lane_fill, in block
+// order), all of block width k with FP32 (f32) or FP64 vectors, in cooperative launches of
+// `blocks` blocks (the lanes' blocks together, at most one per SM).  may_stage: whole tiles
+// through shared memory where the product's rule says so (a launch of one lane; stage_bytes
+// is then the lane's).  pcg_lane_passes: a lane's product work, to share blocks out by.
 struct PcgLane;
+bool pcg_run_supported(int L, int n_up, int k, int f32);
+uint64_t pcg_lane_passes(int L, int n_up, int k, int f32);
 int pcg_lane_fill(PcgLane *lane, const ChainParams &cp, uint32_t n, int k, int f32, const void *dinv, void *r,
-                  void *p, void *t, void *w, const PcgDev &pd, uint32_t *round0, uint32_t *row0);
-int pcg_batch_step(int f32, const PcgLane *lanes_dev, int nlanes, int k, uint32_t rounds, uint32_t rows,
-                   cudaStream_t st);
+                  void *p, void *t, void *w, const PcgDev &pd, uint32_t block0, uint32_t max_blocks, bool may_stage);
+int pcg_run(int f32, const PcgLane *one, const PcgLane *lanes_dev, int nlanes, int k, uint32_t blocks,
+            uint32_t stage_bytes, int steps, cudaStream_t st);
 
 uint32_t host_binom(int n, int k);
 

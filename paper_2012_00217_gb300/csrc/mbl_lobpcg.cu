@@ -278,6 +278,12 @@ struct Solver {
     int enqueue_pcg_steps()
     {
         const PcgDev pd = pcg_dev();
+        if (pcg_run_supported(cp.L, cp.n_up, k, mixed)) {
+            PcgLane lane;
+            MBL_TRY(pcg_lane_fill(&lane, cp, (uint32_t)n, k, mixed, b.dinv, b.pr, b.pp, b.pt, b.pw, pd, 0,
+                                  (uint32_t)num_sms(), true));
+            return pcg_run(mixed, &lane, nullptr, 1, k, lane.nblocks, lane.stage_bytes, m, st);
+        }
         for (int it = 0; it < m; ++it) {
             if (mixed)
                 MBL_TRY(pcg_step<float>(cp, (uint32_t)n, k, (const float *)b.dinv, (float *)b.pr, (float *)b.pp,
@@ -744,8 +750,8 @@ extern "C" int mbl_lobpcg_solve_noalloc(const mbl_chain *chain, double sigma, co
 // workspace holds nlanes slots; each lane solves one problem at a time, and every round
 // advances every lane by one LOBPCG iteration on the caller's stream: the steps before
 // and after the preconditioner are enqueued lane by lane, and the m PCG steps of all
-// lanes run as three launches per step over a table of the lanes (pcg_batch_step).  A
-// lane whose problem has converged (or reached max_iter) writes its results and takes
+// lanes run in shared cooperative launches (pcg_run), each lane on its own blocks.  A lane
+// whose problem has converged (or reached max_iter) writes its results and takes
 // the next problem.  The host synchronises once per round and reads each lane's status
 // words.  When no shifts are given, each problem's spectrum bounds are found first by
 // nlanes host threads, one stream and one slot each.
@@ -1122,29 +1128,51 @@ extern "C" int mbl_lobpcg_solve_batched(int nprob, const mbl_chain *chains, cons
         }
         MBL_TRY(join());
         if (nb > 0 && opts->pcg_iters > 0) {
-            // the lanes' table for the batched PCG launches; widths or tile settings without a
-            // tiled kernel (pcg_lane_fill refuses them) run each lane's own PCG launches
-            uint32_t round0 = 0, row0 = 0;
-            int nt = 0, fill = MBL_OK;
-            for (int l = 0; l < ns && fill == MBL_OK; ++l) {
-                Lane &ln = lanes[(size_t)l];
-                if (!ln.body) continue;
-                Solver &s = ln.s;
-                fill = pcg_lane_fill(&table[(size_t)nt++], s.cp, (uint32_t)s.n, k, mixed, s.b.dinv, s.b.pr, s.b.pp,
-                                     s.b.pt, s.b.pw, s.pcg_dev(), &round0, &row0);
+            // each advancing lane's share of the SMs, by its product work (at least one each);
+            // widths or switches without a resident kernel run each lane's own PCG launches
+            std::vector<int> in;
+            std::vector<uint64_t> work;
+            bool fill = true;
+            uint64_t total = 0;
+            for (int l = 0; l < ns; ++l) {
+                if (!lanes[(size_t)l].body) continue;
+                const Solver &s = lanes[(size_t)l].s;
+                fill = fill && pcg_run_supported(s.cp.L, s.cp.n_up, k, mixed);
+                in.push_back(l);
+                work.push_back(pcg_lane_passes(s.cp.L, s.cp.n_up, k, mixed));
+                total += work.back();
             }
-            if (fill == MBL_ERR_ARG) {
+            if (!fill) {
                 MBL_TRY(fork());
-                for (int l = 0; l < ns; ++l)
-                    if (lanes[(size_t)l].body) MBL_TRY(lanes[(size_t)l].s.enqueue_pcg_steps());
+                for (int l : in) MBL_TRY(lanes[(size_t)l].s.enqueue_pcg_steps());
                 MBL_TRY(join());
             } else {
-                MBL_TRY(fill);
-                if (cudaMemcpyAsync(table_dev, table.data(), sizeof(PcgLane) * (size_t)nt, cudaMemcpyHostToDevice,
+                const int sms = num_sms();
+                std::vector<uint32_t> share(in.size());
+                int left = sms;
+                for (size_t i = 0; i < in.size(); ++i) {
+                    share[i] = (uint32_t)std::max<uint64_t>(1, (uint64_t)(sms - (int)in.size()) * work[i] / total);
+                    left -= (int)share[i];
+                }
+                while (left > 0) {  // the rest one by one where a block has most to do
+                    size_t most = 0;
+                    for (size_t i = 1; i < in.size(); ++i)
+                        if (work[i] * share[most] > work[most] * share[i]) most = i;
+                    ++share[most];
+                    --left;
+                }
+                uint32_t block0 = 0;
+                for (size_t i = 0; i < in.size(); ++i) {
+                    Solver &s = lanes[(size_t)in[i]].s;
+                    PcgLane &t = table[i];
+                    MBL_TRY(pcg_lane_fill(&t, s.cp, (uint32_t)s.n, k, mixed, s.b.dinv, s.b.pr, s.b.pp, s.b.pt, s.b.pw,
+                                          s.pcg_dev(), block0, share[i], false));
+                    block0 += t.nblocks;
+                }
+                if (cudaMemcpyAsync(table_dev, table.data(), sizeof(PcgLane) * in.size(), cudaMemcpyHostToDevice,
                                     st) != cudaSuccess)
                     return MBL_ERR_CUDA;
-                for (int step = 0; step < opts->pcg_iters; ++step)
-                    MBL_TRY(pcg_batch_step(mixed, table_dev, nt, k, round0, row0, st));
+                MBL_TRY(pcg_run(mixed, nullptr, table_dev, (int)in.size(), k, block0, 0, opts->pcg_iters, st));
             }
         }
         MBL_TRY(fork());
