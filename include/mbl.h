@@ -371,7 +371,8 @@ int mbl_gap_ratio(int nprob, int m, const double *evals_dev, int64_t ld, double 
  * normalised: lambda is taken relative to its squared norm).  The reduced density matrix
  * is the direct sum over p (up spins on the left) of M_p M_p^T, M_p holding the column's
  * entries with p up spins on the left (rows: left patterns, columns: right patterns); its
- * eigenvalues come from the smaller Gram of each M_p by FP64 Jacobi.  Writes S_dev[nvec]
+ * eigenvalues come from the smaller Gram of each M_p, in FP64 (Householder reduction and
+ * bisection).  Writes S_dev[nvec]
  * (FP64 device memory; NaN for a zero column).  chain->h, delta and periodic are not used.
  * Limit: every Gram side min(C(l_a, p), C(L - l_a, n_up - p)) <= 512 (the half cut up to
  * L = 22), else MBL_ERR_ARG.  Workspace: mbl_entanglement_workspace_size bytes of device

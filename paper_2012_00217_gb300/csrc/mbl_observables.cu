@@ -110,7 +110,7 @@ extern "C" int mbl_gap_ratio(int nprob, int m, const double *evals_dev, int64_t 
     return cudaGetLastError() == cudaSuccess ? MBL_OK : MBL_ERR_CUDA;
 }
 
-// Largest Gram side the entanglement kernels accept (a one-block Jacobi per block).
+// Largest Gram side the entanglement kernels accept.
 static constexpr int64_t kEntMaxSide = 512;
 
 static int ent_check(const mbl_chain *chain, int l_a, int nvec, mbl::EntanglementPlan *pl)

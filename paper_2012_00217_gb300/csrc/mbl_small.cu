@@ -12,6 +12,8 @@
 #include <math.h>
 #include <stdint.h>
 
+#include <algorithm>
+
 #include "mbl_dense.h"
 #include "mbl_device.cuh"
 #include "mbl_internal.h"
@@ -44,16 +46,14 @@ __host__ __device__ inline int pad_ld(int n) { return n | 1; }
 // with |a_pq| <= eps sqrt(|a_pp a_qq|) are skipped (the relative test keeps the small
 // eigenvalues of graded matrices accurate); sweeps stop when one rotates nothing or after
 // max_sweeps.  On exit diag(A) holds the eigenvalues and the columns of V (stride ld)
-// the eigenvectors (WANT_V = false: eigenvalues only, V not touched).  Each warp rotates
-// whole rows / columns of its pairs, lanes striding the other index.  cs, pairs: n + 2
+// the eigenvectors.  Each warp rotates whole rows / columns of its pairs, lanes striding the other index.  cs, pairs: n + 2
 // entries (shared or global memory of this block).
-template <typename T, bool WANT_V = true>
+template <typename T>
 __device__ void dev_jacobi(int n, int ld, T *A, T *V, T *cs, int *pairs, int *s_rot, int max_sweeps)
 {
     const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5, nwarps = nt >> 5;
-    if (WANT_V)
-        for (int i = warp; i < n; i += nwarps)
-            for (int j = lane; j < n; j += 32) V[i * ld + j] = (i == j) ? (T)1 : (T)0;
+    for (int i = warp; i < n; i += nwarps)
+        for (int j = lane; j < n; j += 32) V[i * ld + j] = (i == j) ? (T)1 : (T)0;
     __syncthreads();
     if (n < 2) return;
     const int np = (n + 1) & ~1;
@@ -116,12 +116,10 @@ __device__ void dev_jacobi(int n, int ld, T *A, T *V, T *cs, int *pairs, int *s_
                     const T ap = Aj[p], aq = Aj[q];
                     Aj[p] = c * ap - s * aq;
                     Aj[q] = s * ap + c * aq;
-                    if (WANT_V) {
-                        T *Vj = V + j * ld;
-                        const T vp = Vj[p], vq = Vj[q];
-                        Vj[p] = c * vp - s * vq;
-                        Vj[q] = s * vp + c * vq;
-                    }
+                    T *Vj = V + j * ld;
+                    const T vp = Vj[p], vq = Vj[q];
+                    Vj[p] = c * vp - s * vq;
+                    Vj[q] = s * vp + c * vq;
                 }
             }
             __syncthreads();
@@ -647,12 +645,60 @@ int gather_cols(int k, int nev, const double *V, const int *sel, double *Csel, c
 // M_p[i][c] = v[off_c + i]: i the colex rank of the left pattern among those with p ones,
 // c the colex rank of the right pattern among those with n_up - p ones, off_c the row of
 // the first state with that right pattern (the left p spins lowest).  The reduced density
-// matrix of the left block is the direct sum of the M_p M_p^T.  One block per
-// (vector, p): M_p gathered densely into its workspace, the smaller Gram (M M^T or
-// M^T M, with the same nonzero eigenvalues), its eigenvalues by Jacobi (FP64), and the
-// sums s0 = sum lambda, s1 = sum lambda ln lambda over lambda > 0, in a fixed order.  A
-// second launch forms S = ln N - (sum_p s1) / N with N = sum_p s0 = ||v||^2, so v need
-// not be normalised.
+// matrix of the left block is the direct sum of the M_p M_p^T.  For each (vector, p):
+//   k_ent_gather   M_p, dense, with the index of the smaller Gram innermost;
+//   k_ent_gram     the smaller Gram (M M^T or M^T M, the same nonzero eigenvalues), in
+//                  tiles of 32 x 32 over all SMs;
+//   k_ent_tridiag  Householder reduction to tridiagonal form by a cluster of four blocks;
+//   k_ent_eig      its eigenvalues by bisection on Sturm counts, one lane each, and the
+//                  sum of lambda ln lambda;
+// and k_ent_combine forms S = ln N - (sum lambda ln lambda) / N with N = sum lambda, the
+// trace of the Grams, so v need not be normalised.  Every sum has a fixed order.
+//
+// All of it is bound by the FP64 pipe (two FMA a cycle and SM on GB300).  At L = 20,
+// l_a = 10, 16 vectors, the one-block FP64 Jacobi in L2 that this replaces took 590 ms,
+// about 20 sweeps of n^3 rotations; the reduction needs n^3 FMA once, spread over four SMs
+// a matrix (6.7 ms the whole call).
+
+constexpr int kEntCluster = 4;    // blocks per matrix in the reduction
+constexpr int kEntThreads = 256;  // threads of the gather, Gram and reduction blocks
+constexpr int kEntTile = 32;      // Gram tile edge
+constexpr int kEntSmem = 224 * 1024;  // rows of the reduction kept in shared memory up to this
+
+// The cut's values of p that occur, largest Gram first.
+struct EntCut {
+    int L, n_up, la, np, job0;  // job0: the first (vector, p) of this launch
+    int p[kMaxL + 1];
+    int64_t block_doubles, mmax, dmax;
+};
+
+// One (vector, p): its sizes and its part of the workspace.
+struct EntJob {
+    int vec, p, R, T, d, t, ld;  // d: Gram side, t: the other side
+    bool left;                   // d = R: Gram over the left patterns
+    // off2[d]: the exponent ex, diag and off2 being those of the matrix over 2^ex
+    double *M, *A, *diag, *off2, *sums;
+};
+
+__device__ __forceinline__ EntJob ent_job(const EntCut &cut, int nvec, int job, double *work)
+{
+    EntJob j;
+    const int q = job / nvec;
+    j.vec = job % nvec;
+    j.p = cut.p[q];
+    j.R = (int)__ldg(&g_binom.v[cut.la * kBinomDim + j.p]);
+    j.T = (int)__ldg(&g_binom.v[(cut.L - cut.la) * kBinomDim + cut.n_up - j.p]);
+    j.left = j.R <= j.T;
+    j.d = j.left ? j.R : j.T;
+    j.t = j.left ? j.T : j.R;
+    j.ld = pad_ld(j.d);
+    j.M = work + (int64_t)job * cut.block_doubles;
+    j.A = j.M + cut.mmax;
+    j.diag = j.A + cut.dmax * (int64_t)pad_ld((int)cut.dmax);
+    j.off2 = j.diag + cut.dmax + 2;
+    j.sums = j.off2 + cut.dmax + 2;  // [0] the trace, [1 + g] lambda ln lambda of 32 eigenvalues
+    return j;
+}
 
 EntanglementPlan entanglement_plan(int L, int n_up, int la)
 {
@@ -667,101 +713,301 @@ EntanglementPlan entanglement_plan(int L, int n_up, int la)
         if (T > pl.tmax) pl.tmax = T;
         if (R * T > pl.mmax) pl.mmax = R * T;
     }
-    // M (mmax), A (dmax x pad_ld(dmax)), cs (dmax + 2), pairs and offsets (as doubles)
+    // M (mmax), A (dmax x pad_ld(dmax)), the tridiagonal (2 (dmax + 2)), the sums (1 + dmax / 32)
     pl.block_doubles = pl.mmax + pl.dmax * (int64_t)pad_ld((int)pl.dmax) + 2 * (pl.dmax + 2) + pl.tmax + 8;
     pl.blocks_per_vector = la + 1;
     return pl;
 }
 
-__global__ void __launch_bounds__(kSmallThreads)
-    k_ent_block(int L, int n_up, int la, const double *__restrict__ V, int64_t ldv, double *work,
-                int64_t block_doubles, int64_t mmax, int64_t dmax, double *parts)
+// M[s][g]: g the Gram index (innermost), s the summed index.
+__global__ void __launch_bounds__(kEntThreads) k_ent_gather(EntCut cut, int nvec, const double *__restrict__ V,
+                                                            int64_t ldv, double *work)
 {
     __shared__ uint32_t sb[kBinomDim * kBinomDim];
-    __shared__ int s_rot;
-    __shared__ double s_r0[kSmallThreads / 32], s_r1[kSmallThreads / 32];
     load_binom(sb);
     __syncthreads();
-    const int e = blockIdx.x / (la + 1), p = blockIdx.x % (la + 1);
-    const int lb = L - la, q = n_up - p;
-    double *out = parts + 2 * (int64_t)blockIdx.x;
-    if (q < 0 || q > lb) {  // no state has p up spins on the left
-        if (threadIdx.x == 0) {
-            out[0] = 0.0;
-            out[1] = 0.0;
-        }
-        return;
-    }
-    const int R = (int)binom(sb, la, p), T = (int)binom(sb, lb, q);
-    const bool left = R <= T;  // Gram over the left patterns (d = R), else over the right ones
-    const int d = left ? R : T, ld = pad_ld(d);
-    double *M = work + (int64_t)blockIdx.x * block_doubles;  // R x T, row-major
-    double *A = M + mmax;
-    double *cs = A + dmax * (int64_t)pad_ld((int)dmax);
-    int *pairs = reinterpret_cast<int *>(cs + dmax + 2);
-    uint32_t *off = reinterpret_cast<uint32_t *>(cs + 2 * (dmax + 2));
-    for (int c = threadIdx.x; c < T; c += blockDim.x) {
+    const EntJob j = ent_job(cut, nvec, cut.job0 + (int)blockIdx.y, work);
+    const int lb = cut.L - cut.la, q = cut.n_up - j.p;
+    const double *v = V + j.vec;
+    // a thread per right pattern c and a run of left patterns: the unranking is done once
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarps = gridDim.x * (kEntThreads / 32);
+    for (int c = blockIdx.x * (kEntThreads / 32) + warp; c < j.T; c += nwarps) {
         const uint32_t b = cns_unrank(sb, lb, q, (uint32_t)c);
-        off[c] = cns_rank(sb, (b << la) | ((1u << p) - 1u));
-    }
-    __syncthreads();
-    const double *v = V + e;
-    for (int64_t x = threadIdx.x; x < (int64_t)R * T; x += blockDim.x) {
-        const int i = (int)(x % R), c = (int)(x / R);  // consecutive threads: consecutive rows of a tile
-        M[(int64_t)i * T + c] = v[((int64_t)off[c] + i) * ldv];
-    }
-    __syncthreads();
-    for (int64_t x = threadIdx.x; x < (int64_t)d * d; x += blockDim.x) {
-        const int i = (int)(x / d), j = (int)(x % d);
-        if (j < i) continue;
-        double acc = 0.0;
-        if (left) {
-            const double *mi = M + (int64_t)i * T, *mj = M + (int64_t)j * T;
-            for (int c = 0; c < T; ++c) acc += mi[c] * mj[c];
-        } else {
-            for (int r = 0; r < R; ++r) acc += M[(int64_t)r * T + i] * M[(int64_t)r * T + j];
-        }
-        A[(int64_t)i * ld + j] = acc;
-        A[(int64_t)j * ld + i] = acc;
-    }
-    __syncthreads();
-    dev_jacobi<double, false>(d, ld, A, nullptr, cs, pairs, &s_rot, kMaxSweeps);
-    double s0 = 0.0, s1 = 0.0;
-    for (int i = threadIdx.x; i < d; i += blockDim.x) {
-        const double lam = A[(int64_t)i * ld + i];
-        if (lam > 0.0) {
-            s0 += lam;
-            s1 += lam * log(lam);
-        }
-    }
-    for (int o = 16; o > 0; o >>= 1) {
-        s0 += __shfl_xor_sync(0xffffffffu, s0, o);
-        s1 += __shfl_xor_sync(0xffffffffu, s1, o);
-    }
-    if ((threadIdx.x & 31) == 0) {
-        s_r0[threadIdx.x >> 5] = s0;
-        s_r1[threadIdx.x >> 5] = s1;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double a0 = 0.0, a1 = 0.0;
-        for (int w = 0; w < kSmallThreads / 32; ++w) {
-            a0 += s_r0[w];
-            a1 += s_r1[w];
-        }
-        out[0] = a0;
-        out[1] = a1;
+        const uint32_t off = cns_rank(sb, (b << cut.la) | ((1u << j.p) - 1u));
+        for (int i = lane; i < j.R; i += 32)
+            j.M[j.left ? (int64_t)c * j.R + i : (int64_t)i * j.T + c] = v[((int64_t)off + i) * ldv];
     }
 }
 
-__global__ void k_ent_combine(int nvec, int per, const double *parts, double *S)
+// One 32 x 32 tile (and its mirror image) of a Gram per block, 2 x 2 outputs a thread.
+__global__ void __launch_bounds__(kEntThreads) k_ent_gram(EntCut cut, int nvec, double *work)
+{
+    constexpr int TS = kEntTile, KS = 16;
+    __shared__ double sa[KS][TS], sc[KS][TS];
+    const EntJob j = ent_job(cut, nvec, cut.job0 + (int)blockIdx.y, work);
+    const int d = j.d, nt = (d + TS - 1) / TS;
+    if ((int)blockIdx.x >= nt * (nt + 1) / 2) return;
+    int bi = 0, rem = blockIdx.x;  // tile (bi, bj), bj >= bi
+    while (rem >= nt - bi) rem -= nt - bi++;
+    const int i0 = bi * TS, j0 = (bi + rem) * TS;
+    const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
+    double acc[2][2] = {};
+    for (int s0 = 0; s0 < j.t; s0 += KS) {
+        for (int e = threadIdx.x; e < KS * TS; e += kEntThreads) {
+            const int s = e / TS, g = e % TS;
+            const double *row = j.M + (int64_t)(s0 + s) * d;
+            sa[s][g] = (s0 + s < j.t && i0 + g < d) ? row[i0 + g] : 0.0;
+            sc[s][g] = (s0 + s < j.t && j0 + g < d) ? row[j0 + g] : 0.0;
+        }
+        __syncthreads();
+#pragma unroll
+        for (int s = 0; s < KS; ++s) {
+            const double a0 = sa[s][ty], a1 = sa[s][ty + 16], c0 = sc[s][tx], c1 = sc[s][tx + 16];
+            acc[0][0] += a0 * c0;
+            acc[0][1] += a0 * c1;
+            acc[1][0] += a1 * c0;
+            acc[1][1] += a1 * c1;
+        }
+        __syncthreads();
+    }
+#pragma unroll
+    for (int a = 0; a < 2; ++a)
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+            const int gi = i0 + ty + 16 * a, gj = j0 + tx + 16 * c;
+            if (gi < d && gj < d && gj >= gi) {
+                j.A[(int64_t)gi * j.ld + gj] = acc[a][c];
+                j.A[(int64_t)gj * j.ld + gi] = acc[a][c];
+            }
+        }
+}
+
+__device__ __forceinline__ void cluster_barrier()
+{
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+// The shared-memory address that holds `p` in block `rank` of the cluster.
+__device__ __forceinline__ uint32_t cluster_addr(const void *p, int rank)
+{
+    uint32_t a;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(rank));
+    return a;
+}
+
+__device__ __forceinline__ double cluster_ld(uint32_t addr)
+{
+    double v;
+    asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(addr) : "memory");
+    return v;
+}
+
+__device__ __forceinline__ void cluster_st(uint32_t addr, double v)
+{
+    asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(addr), "d"(v) : "memory");
+}
+
+__device__ __forceinline__ double warp_sum(double x)
+{
+    for (int off = 16; off > 0; off >>= 1) x += __shfl_xor_sync(0xffffffffu, x, off);
+    return x;
+}
+
+// Householder reduction of A to tridiagonal form: step k takes x = row k beyond the diagonal,
+// v = x - alpha e_1 with alpha = -sign(x_1) ||x||, y = A v, and A -= v w^T + w v^T with
+// w = b y - (b^2 (v.y) / 2) v, b = 2 / v.v.  Row i lives in block i mod 4 of the cluster,
+// column-major (thread = row, so a column's rows are read side by side), in shared memory
+// while a block's rows fit there, else in the workspace.  Per step two cluster barriers: y
+// is spread to all blocks, and the next row is read once every row is updated.  The matrix is
+// scaled by the power of two above its trace; an x whose norm beyond x_1 is below 2^-100 of
+// that is taken as zero (squares of a graded matrix' smallest parts would underflow).
+__global__ void __cluster_dims__(kEntCluster, 1, 1) __launch_bounds__(kEntThreads)
+    k_ent_tridiag(EntCut cut, int nvec, double *work, int in_smem)
+{
+    extern __shared__ __align__(16) double ent_raw[];
+    __shared__ double s_b, s_c, s_part[kEntThreads];
+    const int rank = blockIdx.x % kEntCluster;
+    const EntJob j = ent_job(cut, nvec, cut.job0 + (int)(blockIdx.x / kEntCluster), work);
+    const int d = j.d, nr = (d + kEntCluster - 1) / kEntCluster, dmax = (int)cut.dmax;
+    double *v = ent_raw, *w = v + dmax, *y = w + dmax, *rows = y + dmax;
+    // element (own row li, column c) at At[li * si + c * sc]
+    double *At = in_smem ? rows : j.A + rank;
+    const int64_t si = in_smem ? 1 : kEntCluster, sc = in_smem ? nr : j.ld;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    if (warp == 0) {
+        double tr = 0.0;
+        for (int i = lane; i < d; i += 32) tr += j.A[(int64_t)i * j.ld + i];
+        tr = warp_sum(tr);
+        if (lane == 0) s_b = (tr > 0.0 && isfinite(tr)) ? (double)(ilogb(tr) + 1) : 0.0;
+    }
+    __syncthreads();
+    const int ex = (int)s_b;
+    if (rank == 0 && tid == 0) j.off2[d] = s_b;
+    cluster_barrier();  // every block has read the diagonal
+    for (int e = tid; e < nr * d; e += kEntThreads) {
+        const int c = e / nr, li = e - c * nr, i = rank + kEntCluster * li;
+        if (i < d) At[li * si + c * sc] = scalbn(j.A[(int64_t)c * j.ld + i], -ex);
+    }
+    cluster_barrier();
+    // thread = (row group of 32, column segment): rows tid % 32 + 32 * g, segment warp
+    constexpr int SEG = kEntThreads / 32;
+    for (int k = 0; k < d; ++k) {
+        const int owner = k % kEntCluster, lk = k / kEntCluster;
+        // row k of the reduced matrix, from its owner
+        for (int c = k + tid; c < d; c += kEntThreads) {
+            const double x = in_smem ? cluster_ld(cluster_addr(rows + (int64_t)c * nr + lk, owner))
+                                     : __ldcg(j.A + (int64_t)c * j.ld + k);
+            v[c] = x;
+        }
+        __syncthreads();
+        if (rank == 0 && tid == 0) j.diag[k] = v[k];
+        const int m = d - 1 - k;  // order of the trailing matrix
+        if (m == 0) break;
+        if (m == 1) {
+            if (rank == 0 && tid == 0) j.off2[k] = v[k + 1] * v[k + 1];
+        } else {
+            if (warp == 0) {
+                double s = 0.0;
+                for (int c = k + 2 + lane; c < d; c += 32) s += v[c] * v[c];
+                s = warp_sum(s);
+                if (lane == 0) {
+                    const double x1 = v[k + 1];
+                    double b = 0.0, n2 = x1 * x1;
+                    if (s > 0x1p-200) {
+                        n2 += s;
+                        const double v1 = x1 + copysign(sqrt(n2), x1);
+                        b = 2.0 / (s + v1 * v1);
+                        v[k + 1] = v1;
+                    }
+                    s_b = b;
+                    if (rank == 0) j.off2[k] = n2;
+                }
+            }
+            __syncthreads();
+            const double b = s_b;
+            if (b != 0.0) {  // the same in all blocks
+                // y = A v over own rows, SEG column segments
+                const int first = k + 1;
+                for (int g = 0; g < nr; g += 32) {
+                    const int li = g + lane;
+                    if (rank + kEntCluster * (g + 31) <= k) continue;  // a group of finished rows
+                    double acc = 0.0;
+                    if (li < nr)
+                        for (int c = first + warp; c < d; c += SEG) acc += At[li * si + c * sc] * v[c];
+                    s_part[tid] = acc;
+                    __syncthreads();
+                    if (warp == 0 && li < nr && rank + kEntCluster * li < d) {
+                        double t = 0.0;
+#pragma unroll
+                        for (int q = 0; q < SEG; ++q) t += s_part[32 * q + lane];
+                        const int i = rank + kEntCluster * li;
+                        for (int r = 0; r < kEntCluster; ++r) cluster_st(cluster_addr(y + i, r), t);
+                    }
+                    __syncthreads();
+                }
+                cluster_barrier();
+                if (warp == 0) {
+                    double s = 0.0;
+                    for (int c = first + lane; c < d; c += 32) s += v[c] * y[c];
+                    s = warp_sum(s);
+                    if (lane == 0) s_c = 0.5 * b * s;
+                }
+                __syncthreads();
+                const double h = s_c;
+                for (int c = first + tid; c < d; c += kEntThreads) w[c] = b * (y[c] - h * v[c]);
+                __syncthreads();
+                for (int g = 0; g < nr; g += 32) {
+                    const int li = g + lane, i = rank + kEntCluster * li;
+                    if (i > k && i < d) {
+                        const double vi = v[i], wi = w[i];
+                        for (int c = first + warp; c < d; c += SEG) {
+                            double *a = At + li * si + c * sc;
+                            *a = fma(-wi, v[c], fma(-vi, w[c], *a));
+                        }
+                    }
+                }
+            }
+        }
+        cluster_barrier();
+    }
+    cluster_barrier();  // no block leaves while another may read its rows
+}
+
+// Number of eigenvalues of T below x: sign changes of p_i = (a_i - x) p_{i-1} - b_{i-1}^2
+// p_{i-2}.  Three FP64 operations a step and no division; the exponents are brought back by
+// integer operations after each step, and an exact zero stands for -2^-60 p_{i-1} (a_i moved
+// by 2^-60 of the matrix' scale).  ab[i] = (a_i, b_{i-1}^2).
+__device__ __forceinline__ int sturm_count(const double2 *ab, int d, double x)
+{
+    double p0 = 0.0, p1 = 1.0;
+    int cnt = 0;
+    for (int i = 0; i < d; ++i) {
+        const double2 q = ab[i];
+        const double pn = fma(q.x - x, p1, -(q.y * p0));
+        int h = __double2hiint(pn), lo = __double2loint(pn);
+        const int h1 = __double2hiint(p1);
+        if ((((unsigned)h & 0x7ff00000u) == 0u)) {  // zero (or subnormal): see above
+            h = (int)(((unsigned)h1 ^ 0x80000000u) - (60u << 20));
+            lo = 0;
+        }
+        cnt += (int)(((unsigned)(h ^ h1)) >> 31);
+        const int e = (int)(((unsigned)h >> 20) & 0x7ffu) - 1023;  // p_{i-1} has exponent 0
+        p0 = __hiloint2double(h1 - (int)((unsigned)e << 20), __double2loint(p1));
+        p1 = __hiloint2double(h - (int)((unsigned)e << 20), lo);
+    }
+    return cnt;
+}
+
+// Eigenvalues 32 g .. 32 g + 31 of one matrix by one warp: bisection to 2^-60 of its scale.
+// A warp alone on its quarter of an SM has the whole of that quarter's FP64 pipe.
+__global__ void __launch_bounds__(32) k_ent_eig(EntCut cut, int nvec, double *work)
+{
+    extern __shared__ __align__(16) double2 ent_ab[];
+    const EntJob j = ent_job(cut, nvec, cut.job0 + (int)blockIdx.y, work);
+    const int d = j.d, lane = threadIdx.x, idx = blockIdx.x * 32 + lane;
+    if ((int)blockIdx.x * 32 >= d) return;
+    const int ex = (int)j.off2[d];
+    double tr = 0.0;
+    for (int i = lane; i < d; i += 32) tr += j.diag[i];
+    tr = warp_sum(tr);
+    double sum = 0.0;
+    if (!(tr > 0.0) || !isfinite(tr)) {
+        sum = tr == 0.0 ? 0.0 : NAN;
+        if (tr < 0.0) tr = NAN;
+    } else {
+        // scaled by the power of two above the trace: all eigenvalues in [0, 1], up to rounding
+        for (int i = lane; i < d; i += 32) ent_ab[i] = make_double2(j.diag[i], i > 0 ? j.off2[i - 1] : 0.0);
+        __syncwarp();
+        double lo = -0x1p-40, hi = 1.0 + 0x1p-40;
+        for (int it = 0; it < 64; ++it) {
+            const double mid = 0.5 * (lo + hi);
+            const bool open = hi - lo > 0x1p-60 && mid > lo && mid < hi;
+            if (!__any_sync(0xffffffffu, open)) break;
+            const int c = sturm_count(ent_ab, d, mid);
+            if (open) {
+                if (c > idx) hi = mid;
+                else lo = mid;
+            }
+        }
+        const double lam = scalbn(0.5 * (lo + hi), ex);
+        if (idx < d && lam > 0.0) sum = lam * log(lam);
+    }
+    sum = warp_sum(sum);
+    if (lane == 0) {
+        j.sums[1 + blockIdx.x] = sum;
+        if (blockIdx.x == 0) j.sums[0] = scalbn(tr, ex);
+    }
+}
+
+__global__ void k_ent_combine(EntCut cut, int nvec, double *work, double *S)
 {
     const int e = blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= nvec) return;
     double n2 = 0.0, a1 = 0.0;
-    for (int p = 0; p < per; ++p) {
-        n2 += parts[2 * ((int64_t)e * per + p)];
-        a1 += parts[2 * ((int64_t)e * per + p) + 1];
+    for (int q = 0; q < cut.np; ++q) {
+        const EntJob j = ent_job(cut, nvec, q * nvec + e, work);
+        n2 += j.sums[0];
+        for (int g = 0; 32 * g < j.d; ++g) a1 += j.sums[1 + g];
     }
     S[e] = n2 > 0.0 ? log(n2) - a1 / n2 : NAN;
 }
@@ -770,17 +1016,41 @@ int entanglement_launch(int L, int n_up, int la, int nvec, const double *V, int6
                         size_t work_bytes, cudaStream_t st)
 {
     const EntanglementPlan pl = entanglement_plan(L, n_up, la);
-    const int64_t nblk = (int64_t)nvec * pl.blocks_per_vector;
     const size_t need = entanglement_work_bytes(pl, nvec);
     if (work_bytes < need) return MBL_ERR_WORKSPACE;
     double *w = (double *)(((uintptr_t)work + 255) & ~(uintptr_t)255);
-    double *parts = w + nblk * pl.block_doubles;
+    EntCut cut{};
+    cut.L = L;
+    cut.n_up = n_up;
+    cut.la = la;
+    cut.block_doubles = pl.block_doubles;
+    cut.mmax = pl.mmax;
+    cut.dmax = pl.dmax;
+    auto side = [&](int p) { return std::min(host_binom(la, p), host_binom(L - la, n_up - p)); };
+    for (int p = std::max(0, n_up - (L - la)); p <= std::min(la, n_up); ++p) {
+        int i = cut.np++;
+        for (; i > 0 && side(cut.p[i - 1]) < side(p); --i) cut.p[i] = cut.p[i - 1];
+        cut.p[i] = p;
+    }
+    const unsigned njob = (unsigned)(cut.np * nvec);
+    const int d = (int)pl.dmax, nt = (d + kEntTile - 1) / kEntTile, nr = (d + kEntCluster - 1) / kEntCluster;
+    static const cudaError_t attr = cudaFuncSetAttribute(k_ent_tridiag, cudaFuncAttributeMaxDynamicSharedMemorySize, kEntSmem);
+    if (attr != cudaSuccess) return MBL_ERR_CUDA;
+    const size_t vec_bytes = (size_t)3 * d * sizeof(double), row_bytes = (size_t)nr * d * sizeof(double);
+    const int in_smem = vec_bytes + row_bytes <= (size_t)kEntSmem;
+    for (unsigned done = 0; done < njob; done += 32768u) {  // a grid's second dimension ends at 65,535
+        const unsigned now = std::min(njob - done, 32768u);
+        cut.job0 = (int)done;
+        note_launch(4);
+        k_ent_gather<<<dim3(8, now), kEntThreads, 0, st>>>(cut, nvec, V, ldv, w);
+        k_ent_gram<<<dim3((unsigned)(nt * (nt + 1) / 2), now), kEntThreads, 0, st>>>(cut, nvec, w);
+        k_ent_tridiag<<<now * kEntCluster, kEntThreads, vec_bytes + (in_smem ? row_bytes : 0), st>>>(cut, nvec, w,
+                                                                                                     in_smem);
+        k_ent_eig<<<dim3((unsigned)((d + 31) / 32), now), 32, (size_t)d * sizeof(double2), st>>>(cut, nvec, w);
+        if (cudaGetLastError() != cudaSuccess) return MBL_ERR_CUDA;
+    }
     note_launch();
-    k_ent_block<<<(unsigned)nblk, kSmallThreads, 0, st>>>(L, n_up, la, V, ldv, w, pl.block_doubles, pl.mmax,
-                                                          pl.dmax, parts);
-    if (cudaGetLastError() != cudaSuccess) return MBL_ERR_CUDA;
-    note_launch();
-    k_ent_combine<<<(nvec + 127) / 128, 128, 0, st>>>(nvec, pl.blocks_per_vector, parts, S);
+    k_ent_combine<<<(nvec + 127) / 128, 128, 0, st>>>(cut, nvec, w, S);
     return cudaGetLastError() == cudaSuccess ? MBL_OK : MBL_ERR_CUDA;
 }
 
