@@ -68,6 +68,7 @@ enum ApplyMode {
     kPlain = 0,    // Y = (H - sigma) X
     kPcgT = 1,     // t = (H - sigma) p; accumulate t.t per column; finish alpha = rz / t.t
     kPcgQ = 2,     // q = (H - sigma) t; r -= alpha q; accumulate r.(dinv r); finish beta
+    kDot = 3,      // w = (H - sigma) v; accumulate v.w per column (resident Lanczos)
 };
 
 // Per-column PCG scalars (FP64), laid out as arrays of kMaxK.
@@ -802,7 +803,17 @@ __device__ __forceinline__ void tile_row_pass(const ChainParams &cp, int B, cons
                 return;
             }
         }
-        finish_row<T, V, MODE>(acc, 0, r, Y, ldy, R, dinv, col, alpha, part, (T *)ps_w, (const T *)ps_p);
+        if constexpr (MODE == kDot) {
+            Vec<T, V> y;
+#pragma unroll
+            for (int v = 0; v < V; ++v) {
+                y.v[v] = acc[v];
+                part[v] += x.v[v] * acc[v];
+            }
+            stv<T, V>(Y + (int64_t)r * ldy + col, y);
+        } else {
+            finish_row<T, V, MODE>(acc, 0, r, Y, ldy, R, dinv, col, alpha, part, (T *)ps_w, (const T *)ps_p);
+        }
     }
 }
 
@@ -2266,12 +2277,13 @@ __device__ __forceinline__ bool lane_column_sums(double *buf, unsigned &target)
     const int nb = (int)sm.lane.nblocks, bl = (int)(blockIdx.x - sm.lane.block0);
     static_assert(kRunWarps == 24 && 8 * K <= kRunThreads, "three warps' sums for each of eight threads");
     __syncthreads();
-    if (threadIdx.x < 8 * K) {
+    if (threadIdx.x < (8 * K + 31) / 32 * 32) {  // whole warps
         const int c = threadIdx.x >> 3, j = threadIdx.x & 7;
-        ColSum<T> s = (ColSum<T>(sm.red[j][c]) + ColSum<T>(sm.red[j + 8][c])) + ColSum<T>(sm.red[j + 16][c]);
+        ColSum<T> s((T)0);
+        if (c < K) s = (ColSum<T>(sm.red[j][c]) + ColSum<T>(sm.red[j + 8][c])) + ColSum<T>(sm.red[j + 16][c]);
 #pragma unroll
         for (int off = 4; off > 0; off >>= 1) s = s + s.shfl(off);
-        if (j == 0) s.store(buf + c * nb + bl);
+        if (j == 0 && c < K) s.store(buf + c * nb + bl);
     }
     if (!lane_barrier<ASYNC>(sm, target)) return false;
     constexpr int CPW = (K + kRunWarps - 1) / kRunWarps, BPL = kRunMaxBlocks / 32;
@@ -2372,8 +2384,8 @@ __device__ __forceinline__ void run_cache_jobs(RunShared<T> &sm, const RunShare 
 }
 
 // The product of this block's jobs: Y = (H - sigma) X and, per column, the warp's sum of
-// y.y (kPcgT), or q = (H - sigma) X, R -= alpha q and the sum of R.(M^-1 R) (kPcgQ), into
-// sm.red.  Staged: a group of 256 threads takes whole tiles, one at a time: the other groups
+// y.y (kPcgT) or x.y (kDot), or q = (H - sigma) X, R -= alpha q and the sum of R.(M^-1 R)
+// (kPcgQ), into sm.red.  Staged: a group of 256 threads takes whole tiles, one at a time: the other groups
 // work while its copy is in flight, and a second buffer would come out of the L1 that loads
 // in flight need (L = 20, k = 32: 105 us a step with two buffers, 93 with one).  Else a
 // warp takes a chunk of a tile.
@@ -2390,8 +2402,8 @@ __device__ __noinline__ void run_product()
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, grp = lane / G, col = (lane % G) * V;
     const int B = Ln.B, H = cp.L - B;
     const T hdelta = cp_half_delta<T>(cp);
-    T *X = as_global<T>(MODE == kPcgT ? Ln.p : Ln.t);
-    T *Y = MODE == kPcgT ? as_global<T>(Ln.t) : nullptr;
+    T *X = as_global<T>(MODE == kPcgQ ? Ln.t : Ln.p);
+    T *Y = MODE != kPcgQ ? as_global<T>(Ln.t) : nullptr;
     T *R = MODE == kPcgQ ? as_global<T>(Ln.r) : nullptr;
     const T *dinv = as_global<T>(const_cast<void *>(Ln.dinv));
     const LowRec *tbl = g_lowtab + lowtab_base(B);
@@ -2598,28 +2610,15 @@ __device__ __noinline__ void run_update(uint32_t row_b, uint32_t row_e, uint32_t
     if (W_TMEM) tmem_wait_st();
 }
 
-template <typename T, int K, bool STAGED>
-__global__ void __launch_bounds__(kRunThreads, 1)
-    k_pcg_run(const __grid_constant__ PcgLane one, const PcgLane *lanes, int nlanes, int steps)
+// What a block keeps for the whole launch: its lane, the tables, the classes of tiles.
+template <typename T, bool STAGED>
+__device__ __forceinline__ void run_setup(const PcgLane *src)
 {
     RunShared<T> &sm = run_shared<T>();
     const PcgLane &Ln = sm.lane;
-    {
-        // the lane this block serves
-        const PcgLane *src = &one;
-        if (lanes) {
-            int lo = 0, hi = nlanes - 1;
-            while (lo < hi) {
-                const int mid = (lo + hi + 1) >> 1;
-                if (lanes[mid].block0 <= blockIdx.x) lo = mid;
-                else hi = mid - 1;
-            }
-            src = lanes + lo;
-        }
-        const int *s = reinterpret_cast<const int *>(src);
-        int *d = reinterpret_cast<int *>(&sm.lane);
-        for (int i = threadIdx.x; i < (int)(sizeof(PcgLane) / sizeof(int)); i += kRunThreads) d[i] = s[i];
-    }
+    const int *s = reinterpret_cast<const int *>(src);
+    int *d = reinterpret_cast<int *>(&sm.lane);
+    for (int i = threadIdx.x; i < (int)(sizeof(PcgLane) / sizeof(int)); i += kRunThreads) d[i] = s[i];
     load_binom(sm.binom);
     if (STAGED && threadIdx.x < kRunSubs) mbar_init(&sm.mbar[threadIdx.x], 1);
     if (threadIdx.x < kRunWarps) sm.parity[threadIdx.x] = 0;
@@ -2650,12 +2649,45 @@ __global__ void __launch_bounds__(kRunThreads, 1)
         }
         sm.ncls = n;
     }
-    if (threadIdx.x >= 64 && threadIdx.x < 64 + K) {
-        const int c = threadIdx.x - 64;
-        sm.rz[c] = ColSum<T>::of(Ln.rz[c]);
-        sm.active[c] = Ln.active[c];
-    }
     __syncthreads();
+}
+
+// The last block of a lane to leave puts the barrier words back to zero.
+__device__ __forceinline__ void run_leave(const PcgLane &Ln)
+{
+    if (Ln.nblocks > 1 && threadIdx.x == 0) {
+        __threadfence();
+        if (atomicAdd(Ln.counter + 2, 1u) == Ln.nblocks - 1u) {
+            Ln.counter[1] = 0u;
+            Ln.counter[2] = 0u;
+        }
+    }
+}
+
+template <typename T, int K, bool STAGED>
+__global__ void __launch_bounds__(kRunThreads, 1)
+    k_pcg_run(const __grid_constant__ PcgLane one, const PcgLane *lanes, int nlanes, int steps)
+{
+    RunShared<T> &sm = run_shared<T>();
+    const PcgLane &Ln = sm.lane;
+    {
+        // the lane this block serves
+        const PcgLane *src = &one;
+        if (lanes) {
+            int lo = 0, hi = nlanes - 1;
+            while (lo < hi) {
+                const int mid = (lo + hi + 1) >> 1;
+                if (lanes[mid].block0 <= blockIdx.x) lo = mid;
+                else hi = mid - 1;
+            }
+            src = lanes + lo;
+        }
+        run_setup<T, STAGED>(src);
+    }
+    if (threadIdx.x < K) {
+        sm.rz[threadIdx.x] = ColSum<T>::of(Ln.rz[threadIdx.x]);
+        sm.active[threadIdx.x] = Ln.active[threadIdx.x];
+    }
     const uint32_t nb = Ln.nblocks, bl = blockIdx.x - Ln.block0;
     const uint32_t row_b = (uint32_t)((uint64_t)Ln.n * bl / nb), row_e = (uint32_t)((uint64_t)Ln.n * (bl + 1) / nb);
     // w in tensor memory when the block's rows fit there
@@ -2717,14 +2749,82 @@ __global__ void __launch_bounds__(kRunThreads, 1)
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     if (w_tmem && threadIdx.x < 32)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512) : "memory");
-    // the last block to leave puts the barrier words back to zero
-    if (nb > 1 && threadIdx.x == 0) {
-        __threadfence();
-        if (atomicAdd(Ln.counter + 2, 1u) == nb - 1u) {
-            Ln.counter[1] = 0u;
-            Ln.counter[2] = 0u;
+    run_leave(Ln);
+}
+
+// Resident Lanczos: steps j0 .. j0 + steps - 1 of the recurrence
+//   w = H v_j,  alpha_j = v_j.w,  w -= alpha_j v_j + beta_{j-1} v_{j-1},  beta_j = ||w||
+// on vectors kept unnormalised (v_j = u_j / beta_{j-1}), two phases and two barriers a step:
+// w = H u_j with u_j.w, then u_{j+1} = w / beta_{j-1} - (alpha_j / beta_{j-1}) u_j -
+// (beta_{j-1} / beta_{j-2}) u_{j-1}, in place of u_{j-1}'s successor, with its norm.  The
+// four launches of a step that this replaces (product, dot product, update, scale) took
+// 69 us at L = 20, most of it between and at the ends of the launches.  lane: p, t and r
+// hold u_j, the next vector and u_{j-1} of step j0; alpha, beta: the recurrence's
+// coefficients; rz: the norm of u_0.
+__global__ void __launch_bounds__(kRunThreads, 1) k_lz_run(const __grid_constant__ PcgLane one, int j0, int steps)
+{
+    RunShared<double> &sm = run_shared<double>();
+    PcgLane &Ln = sm.lane;
+    run_setup<double, false>(&one);
+    run_cache_jobs<double>(sm, run_share<false>(Ln), false);
+    const uint32_t nb = Ln.nblocks, bl = blockIdx.x - Ln.block0;
+    const uint32_t row_b = (uint32_t)((uint64_t)Ln.n * bl / nb), row_e = (uint32_t)((uint64_t)Ln.n * (bl + 1) / nb);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    __shared__ double s_c[3];
+    double inv = 0.0, inv_up = 0.0, beta_up = 0.0;  // thread 0: 1 / |u_j|, 1 / |u_{j-1}|, beta_{j-1}
+    if (threadIdx.x == 0) {
+        auto recip = [](double x) { return x > 0.0 ? 1.0 / x : 0.0; };
+        inv = recip(j0 > 0 ? Ln.beta[j0 - 1] : Ln.rz[0]);
+        if (j0 > 0) {
+            inv_up = recip(j0 > 1 ? Ln.beta[j0 - 2] : Ln.rz[0]);
+            beta_up = Ln.beta[j0 - 1];
         }
     }
+    __syncthreads();
+    unsigned target = 0;
+    bool ok = true;
+    int j = j0;
+#pragma unroll 1
+    for (; j < j0 + steps; ++j) {
+        run_product<double, 1, kDot, false>();
+        if (!(ok = lane_column_sums<double, 1, false>(Ln.partials, target))) break;
+        if (threadIdx.x == 0) {
+            const double a = sm.tot[0].value() * inv * inv;
+            if (bl == 0) Ln.alpha[j] = a;
+            s_c[0] = inv;
+            s_c[1] = a * inv;
+            s_c[2] = beta_up * inv_up;
+        }
+        __syncthreads();
+        double acc = 0.0;
+        {
+            const double c0 = s_c[0], c1 = s_c[1], c2 = s_c[2];
+            double *w = as_global<double>(Ln.t);
+            const double *u = as_global<double>(Ln.p), *up = as_global<double>(Ln.r);
+            for (uint32_t i = row_b + threadIdx.x; i < row_e; i += kRunThreads) {
+                const double x = c0 * w[i] - c1 * u[i] - c2 * up[i];
+                w[i] = x;
+                acc += x * x;
+            }
+        }
+        for (int off = 16; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
+        if (lane == 0) sm.red[warp][0] = acc;
+        if (!(ok = lane_column_sums<double, 1, false>(Ln.partials + nb, target))) break;
+        if (threadIdx.x == 0) {
+            const double s = sm.tot[0].value(), b = sqrt(s);
+            if (bl == 0) Ln.beta[j] = b;
+            inv_up = inv;
+            inv = b > 0.0 ? 1.0 / b : 0.0;
+            beta_up = b;
+            void *up = Ln.r;  // the vectors change roles
+            Ln.r = Ln.p;
+            Ln.p = Ln.t;
+            Ln.t = up;
+        }
+        __syncthreads();
+    }
+    if (!ok && threadIdx.x == 0) Ln.beta[j] = NAN;  // the host takes it as MBL_ERR_NUMERIC
+    run_leave(Ln);
 }
 
 // Generic-k version of the PCG product kernels (one warp per row, lanes stride the
@@ -3405,12 +3505,34 @@ bool pcg_run_supported(int L, int n_up, int k, int f32)
     return o != 4 && o != 5 && lb == 0;
 }
 
+// The lane's blocks and items for chunks of tiles: as many passes an item as give the fewest
+// rounds of passes, an item's set-up counted as half a pass.
+static void run_split(PcgLane &o, int k, size_t es, uint32_t max_blocks)
+{
+    const int L = o.cp.L, n_up = o.cp.n_up;
+    const uint32_t rpw = run_rows_per_pass(k, es);
+    const uint64_t passes = run_items(L, n_up, o.B, rpw);
+    const uint64_t need = (passes + kRunSpread - 1) / kRunSpread;
+    o.nblocks = (uint32_t)(need < max_blocks ? need : max_blocks);
+    const uint64_t warps = (uint64_t)o.nblocks * kRunWarps;
+    uint32_t best = 1;
+    double best_cost = 0.0;
+    for (uint32_t q = 1; q <= 16; ++q) {
+        const uint64_t items = run_items(L, n_up, o.B, rpw * q);
+        const double cost = (double)((items + warps - 1) / warps) * (q + 0.5);
+        if (q == 1 || cost < best_cost) {
+            best = q;
+            best_cost = cost;
+        }
+    }
+    o.chunk = rpw * best;
+}
+
 int pcg_lane_fill(PcgLane *Ln, const ChainParams &cp, uint32_t n, int k, int f32, const void *dinv, void *r,
                   void *p, void *t, void *w, const PcgDev &pd, uint32_t block0, uint32_t max_blocks, bool may_stage)
 {
     const size_t es = f32 ? 4 : 8;
     if (!pcg_run_supported(cp.L, cp.n_up, k, f32) || max_blocks < 1) return MBL_ERR_ARG;
-    const uint32_t rpw = run_rows_per_pass(k, es);
     PcgLane o{};
     o.cp = cp;
     o.dinv = dinv;
@@ -3437,27 +3559,53 @@ int pcg_lane_fill(PcgLane *Ln, const ChainParams &cp, uint32_t n, int k, int f32
         o.nblocks = max_blocks;
     } else {
         o.B = tile_bits_for(cp.L, k, es);
-        const uint64_t passes = run_items(cp.L, cp.n_up, o.B, rpw);
-        const uint64_t need = (passes + kRunSpread - 1) / kRunSpread;
-        o.nblocks = (uint32_t)(need < max_blocks ? need : max_blocks);
-        const uint64_t warps = (uint64_t)o.nblocks * kRunWarps;
-        uint32_t best = 1;
-        double best_cost = 0.0;
-        // passes per item: the fewest rounds of passes, an item's set-up counted as half a pass
-        for (uint32_t q = 1; q <= 16; ++q) {
-            const uint64_t items = run_items(cp.L, cp.n_up, o.B, rpw * q);
-            const double cost = (double)((items + warps - 1) / warps) * (q + 0.5);
-            if (q == 1 || cost < best_cost) {
-                best = q;
-                best_cost = cost;
-            }
-        }
-        o.chunk = rpw * best;
+        run_split(o, k, es, max_blocks);
     }
     if (ensure_lowtab(o.B) != MBL_OK) return MBL_ERR_CUDA;
     o.items = (uint32_t)run_items(cp.L, cp.n_up, o.B, o.chunk);
     *Ln = o;
     return MBL_OK;
+}
+
+// Resident Lanczos: the default switches of width-1 FP64 products, three vectors within L2.
+bool lanczos_run_supported(int L, int n_up)
+{
+    return (double)host_binom(L, n_up) * 8.0 * 3.0 <= kRunL2Bytes && tile_bits_for(L, 1, 8) >= 2 &&
+           g_schedule[1][kslot(1)] == 0 && g_lane_bytes[1][kslot(1)] == 0;
+}
+
+int lanczos_run(const ChainParams &cp, uint32_t n, double *u, double *next, double *up, double *alpha, double *beta,
+                double *norm0, double *partials, unsigned *counter, uint32_t max_blocks, int j0, int steps,
+                cudaStream_t st)
+{
+    PcgLane o{};
+    o.cp = cp;
+    o.p = u;
+    o.t = next;
+    o.r = up;
+    o.alpha = alpha;
+    o.beta = beta;
+    o.rz = norm0;
+    o.partials = partials;
+    o.counter = counter;
+    o.n = n;
+    o.B = tile_bits_for(cp.L, 1, 8);
+    if (o.B < 2 || ensure_lowtab(o.B) != MBL_OK) return MBL_ERR_CUDA;
+    if (max_blocks > (uint32_t)kRunMaxBlocks) max_blocks = kRunMaxBlocks;
+    run_split(o, 1, 8, max_blocks < 1 ? 1 : max_blocks);
+    o.items = (uint32_t)run_items(cp.L, cp.n_up, o.B, o.chunk);
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(o.nblocks);
+    cfg.blockDim = dim3(kRunThreads);
+    cfg.dynamicSmemBytes = run_stage_offset<double>();
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeCooperative;
+    at[0].val.cooperative = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    note_launch();
+    return cudaLaunchKernelEx(&cfg, k_lz_run, o, j0, steps) == cudaSuccess ? MBL_OK : MBL_ERR_CUDA;
 }
 
 template <typename T, int K, bool STAGED>

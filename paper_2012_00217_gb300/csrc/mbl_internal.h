@@ -28,10 +28,12 @@ void note_launch(int64_t count = 1);
 void set_capturing(bool on);
 
 int num_sms();
-// Spectrum bounds by FP64 Lanczos on H (mbl_lanczos.cu); X0: start vector in column 0 (ld).
+// Spectrum bounds by FP64 Lanczos on H (mbl_lanczos.cu); X0: start vector in column 0 (ld);
+// max_blocks: the SMs this call may fill (fewer when several run side by side).
 size_t lanczos_workspace_bytes(int64_t n);
 int lanczos_bounds(const ChainParams &cp, int64_t n, const double *X0, int64_t ldx0, double tol, int max_iter,
-                   void *ws, size_t ws_bytes, double *emin, double *emax, int *iters, cudaStream_t st);
+                   void *ws, size_t ws_bytes, double *emin, double *emax, int *iters, int max_blocks,
+                   cudaStream_t st);
 // Upload the low-pattern tables of every tile width usable at chain length L.
 int ensure_lowtabs_for(int L);
 int make_chain_params(const mbl_chain *chain, double sigma, ChainParams *cp);
@@ -66,6 +68,12 @@ bool pcg_run_supported(int L, int n_up, int k, int f32);
 uint64_t pcg_lane_passes(int L, int n_up, int k, int f32);
 int pcg_lane_fill(PcgLane *lane, const ChainParams &cp, uint32_t n, int k, int f32, const void *dinv, void *r,
                   void *p, void *t, void *w, const PcgDev &pd, uint32_t block0, uint32_t max_blocks, bool may_stage);
+// Resident Lanczos steps j0 .. j0 + steps - 1 in one cooperative launch (mbl_apply.cu says
+// which vector is which); partials: >= 2 max_blocks doubles, counter: four zeroed words.
+bool lanczos_run_supported(int L, int n_up);
+int lanczos_run(const ChainParams &cp, uint32_t n, double *u, double *next, double *up, double *alpha, double *beta,
+                double *norm0, double *partials, unsigned *counter, uint32_t max_blocks, int j0, int steps,
+                cudaStream_t st);
 int pcg_run(int f32, const PcgLane *one, const PcgLane *lanes_dev, int nlanes, int k, uint32_t blocks,
             uint32_t stage_bytes, int steps, cudaStream_t st);
 

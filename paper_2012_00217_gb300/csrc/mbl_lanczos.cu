@@ -3,7 +3,8 @@
 // recurrence on H:
 //   w = H v_j,  alpha_j = v_j^T w,  w -= alpha_j v_j + beta_{j-1} v_{j-1},
 //   beta_j = ||w||,  v_{j+1} = w / beta_j,
-// one block product of width 1 and three small streaming kernels per step.  Both ends come
+// in one cooperative launch per 20 steps while the vectors stay in L2 (lanczos_run), else one
+// block product of width 1 and three small streaming kernels per step.  Both ends come
 // from the same tridiagonal T_m = tridiag(beta, alpha, beta): its extreme eigenvalues by
 // Sturm bisection, and the residual of each extreme Ritz pair as beta_m |y_m| (y the
 // eigenvector of T_m, by inverse iteration).  No reorthogonalisation: the extreme Ritz
@@ -190,7 +191,8 @@ size_t lanczos_workspace_bytes(int64_t n)
 }
 
 int lanczos_bounds(const ChainParams &cp, int64_t n, const double *X0, int64_t ldx0, double tol, int max_iter,
-                   void *ws, size_t ws_bytes, double *emin, double *emax, int *iters, cudaStream_t st)
+                   void *ws, size_t ws_bytes, double *emin, double *emax, int *iters, int max_blocks,
+                   cudaStream_t st)
 {
     if (ws_bytes < lanczos_workspace_bytes(n)) return MBL_ERR_WORKSPACE;
     if (max_iter > kLzMaxSteps) max_iter = kLzMaxSteps;
@@ -210,14 +212,17 @@ int lanczos_bounds(const ChainParams &cp, int64_t n, const double *X0, int64_t l
     p += (size_t)(4 * num_sms() + 8) * sizeof(double);
     d.counter = (unsigned *)p;
     double *nrm0 = (double *)(p + 64);
-    if (cudaMemsetAsync(d.counter, 0, sizeof(unsigned), st) != cudaSuccess ||
+    if (cudaMemsetAsync(d.counter, 0, 4 * sizeof(unsigned), st) != cudaSuccess ||
         cudaMemsetAsync(d.v[0], 0, (size_t)n * sizeof(double), st) != cudaSuccess)
         return MBL_ERR_CUDA;
     // v_0 = X0[:, 0] / ||X0[:, 0]||;  v_prev = 0
     note_launch();
     k_lz_start<<<grid, kLzThreads, 0, st>>>(X0, ldx0, d.v[1], n, nrm0, d.part, d.counter);
-    note_launch();
-    k_lz_scale<<<grid, kLzThreads, 0, st>>>(d.v[1], n, nrm0);
+    const bool resident = lanczos_run_supported(cp.L, cp.n_up);
+    if (!resident) {
+        note_launch();
+        k_lz_scale<<<grid, kLzThreads, 0, st>>>(d.v[1], n, nrm0);
+    }
     if (cudaGetLastError() != cudaSuccess) return MBL_ERR_CUDA;
 
     std::vector<double> a, b;
@@ -225,23 +230,33 @@ int lanczos_bounds(const ChainParams &cp, int64_t n, const double *X0, int64_t l
     int m = 0;
     double lo = 0.0, hi = 0.0;
     bool done = false, ok = false;
-    for (int j = 0; j < max_iter && !done; ++j) {
-        const int rc = apply_device(cp, MBL_F64, d.v[iv], 1, d.v[iw], 1, (uint32_t)n, 1, st);
-        if (rc != MBL_OK) return rc;
-        note_launch();
-        k_lz_alpha<<<grid, kLzThreads, 0, st>>>(d.v[iv], d.v[iw], n, d.alpha + j, d.part, d.counter);
-        note_launch();
-        k_lz_update<<<grid, kLzThreads, 0, st>>>(d.v[iv], d.v[ip], d.v[iw], n, d.alpha + j,
-                                                  j > 0 ? d.beta + j - 1 : nullptr, d.beta + j, d.part, d.counter);
-        note_launch();
-        k_lz_scale<<<grid, kLzThreads, 0, st>>>(d.v[iw], n, d.beta + j);
-        if (cudaGetLastError() != cudaSuccess) return MBL_ERR_CUDA;
-        const int t = ip;
-        ip = iv;
-        iv = iw;
-        iw = t;
-        m = j + 1;
-        if (m % kLzCheckEvery != 0 && m != max_iter) continue;
+    while (m < max_iter && !done) {
+        const int steps = std::min(kLzCheckEvery, max_iter - m);
+        if (resident) {
+            const int rc = lanczos_run(cp, (uint32_t)n, d.v[iv], d.v[iw], d.v[ip], d.alpha, d.beta, nrm0, d.part,
+                                       d.counter, (uint32_t)max_blocks, m, steps, st);
+            if (rc != MBL_OK) return rc;
+        }
+        for (int j = m; j < m + steps; ++j) {
+            if (!resident) {
+                const int rc = apply_device(cp, MBL_F64, d.v[iv], 1, d.v[iw], 1, (uint32_t)n, 1, st);
+                if (rc != MBL_OK) return rc;
+                note_launch();
+                k_lz_alpha<<<grid, kLzThreads, 0, st>>>(d.v[iv], d.v[iw], n, d.alpha + j, d.part, d.counter);
+                note_launch();
+                k_lz_update<<<grid, kLzThreads, 0, st>>>(d.v[iv], d.v[ip], d.v[iw], n, d.alpha + j,
+                                                          j > 0 ? d.beta + j - 1 : nullptr, d.beta + j, d.part,
+                                                          d.counter);
+                note_launch();
+                k_lz_scale<<<grid, kLzThreads, 0, st>>>(d.v[iw], n, d.beta + j);
+                if (cudaGetLastError() != cudaSuccess) return MBL_ERR_CUDA;
+            }
+            const int t = ip;
+            ip = iv;
+            iv = iw;
+            iw = t;
+        }
+        m += steps;
         a.resize(m);
         b.resize(m);
         if (cudaMemcpyAsync(a.data(), d.alpha, m * sizeof(double), cudaMemcpyDeviceToHost, st) != cudaSuccess ||

@@ -681,7 +681,7 @@ extern "C" int mbl_spectrum_bounds(const mbl_chain *chain, int k, double tol, in
     double lo = 0.0, hi = 0.0;
     const int64_t n = mbl_basis_size(chain->L, chain->n_up);
     rc = lanczos_bounds(cp, n, X0_dev, k, tol, max_iter, workspace_dev, workspace_bytes, &lo, &hi, iters_host,
-                        (cudaStream_t)stream);
+                        num_sms(), (cudaStream_t)stream);
     if (rc != MBL_OK && rc != MBL_ERR_NOT_CONVERGED) return rc;
     if (emin_host) *emin_host = lo;
     if (emax_host) *emax_host = hi;
@@ -818,7 +818,7 @@ int batch_bounds(int nprob, const mbl_chain *chains, const double *X0_dev, const
             if (r1 == MBL_OK) r1 = ensure_lowtabs_for(ch.L);
             if (r1 == MBL_OK)
                 r1 = lanczos_bounds(cpb, mbl_basis_size(ch.L, ch.n_up), X0_dev + off_x[i], k, kBatchBoundsTol, 1000,
-                                    ws, slot, &lo, &hi, &it, st);
+                                    ws, slot, &lo, &hi, &it, std::max(1, num_sms() / nth), st);
             if (r1 != MBL_OK && r1 != MBL_ERR_NOT_CONVERGED) {
                 int expect = MBL_OK;
                 first_error.compare_exchange_strong(expect, r1);

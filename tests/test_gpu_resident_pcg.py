@@ -67,3 +67,21 @@ def test_batch_with_w_outside_tensor_memory(mbl):
     for i in (0, 31, 63):
         single, _, _, _ = mbl.lobpcg_solve(chains[i], sigmas[i], opts, X0[i * n:(i + 1) * n].contiguous(), one)
         assert np.abs(single - evals[i]).max() <= 1e-9 * 30.0
+
+
+# the resident Lanczos kernel: one block, several, off-centre sectors, an invariant subspace
+# (n_up = 1: it ends at step n), a last launch of fewer steps.  1e-9: the residual bound of the
+# call, 1e-7 relative, squared over a gap of the spectrum's ends
+@pytest.mark.parametrize("L,n_up,periodic,max_iter", [
+    (4, 2, True, 400), (6, 3, False, 400), (9, 1, True, 9), (10, 4, True, 400), (12, 6, False, 133), (13, 5, True, 400)])
+def test_resident_lanczos_matches_dense(mbl, L, n_up, periodic, max_iter):
+    h = wl.fields(L, 5.0, 60 + L)
+    ev = np.linalg.eigvalsh(ham.dense_sector(ham.Chain(L, h, n_up=n_up, periodic=periodic)))
+    chain = mbl.make_chain(L, h, 1.0, periodic, n_up)
+    n = ham.sector_dim(L, n_up)
+    X0 = torch.from_numpy(wl.block(n, 2, 8)).to(DEV)
+    ws = torch.empty(mbl.bounds_workspace_size(chain, 2), dtype=torch.uint8, device=DEV)
+    lo, hi, steps = mbl.spectrum_bounds(chain, X0, ws, tol=1e-7, max_iter=max_iter)
+    scale = max(abs(ev[0]), abs(ev[-1]))
+    assert abs(lo - ev[0]) <= 1e-9 * scale and abs(hi - ev[-1]) <= 1e-9 * scale and 1 <= steps <= max_iter
+    assert mbl.spectrum_bounds(chain, X0, ws, tol=1e-7, max_iter=max_iter) == (lo, hi, steps)
