@@ -53,9 +53,9 @@ struct WideRowLayout {
     static constexpr int V = kBytes >= LB ? LB / (int)sizeof(T) : K;
     static constexpr int G = K / V;
     static_assert(G >= 1 && G <= 32 && (G & (G - 1)) == 0, "unsupported row width");
-    // rows per work item of the tiled product: at least MBL_CH_PASSES row-passes of the
-    // warp (32 / G rows each) and at least MBL_CH_MIN rows, so the per-tile setup of an
-    // item (tile offset, high-bond shifts) is spread over enough rows
+    // rows per work item of the tiled product, at most (chunk_rows): MBL_CH_PASSES row-passes
+    // of the warp (32 / G rows each) and at least MBL_CH_MIN rows, so the per-tile setup of
+    // an item (tile offset, high-bond shifts) is spread over enough rows
     static constexpr int CH = (MBL_CH_PASSES * (32 / G) > MBL_CH_MIN) ? MBL_CH_PASSES * (32 / G) : MBL_CH_MIN;
 };
 
@@ -818,7 +818,7 @@ __device__ __forceinline__ void tile_row_pass(const ChainParams &cp, int B, cons
 }
 
 template <typename T, int K, int MODE, int LB>
-__global__ void __launch_bounds__(kThreads, MBL_TILED_MIN_BLOCKS) k_apply_tiled(ChainParams cp, int B,
+__global__ void __launch_bounds__(kThreads, MBL_TILED_MIN_BLOCKS) k_apply_tiled(ChainParams cp, int B, uint32_t CH,
                                                                                const T *__restrict__ X, int64_t ldx,
                                                                                T *__restrict__ Y, int64_t ldy,
                                                                                T *__restrict__ R,
@@ -826,7 +826,7 @@ __global__ void __launch_bounds__(kThreads, MBL_TILED_MIN_BLOCKS) k_apply_tiled(
                                                                                PcgScalars ps, Reduce rd)
 {
     using Lay = WideRowLayout<T, K, LB>;
-    constexpr int V = Lay::V, G = Lay::G, RPW = 32 / G, CH = Lay::CH;
+    constexpr int V = Lay::V, G = Lay::G, RPW = 32 / G;
     // neighbour loads issued together: 128 bytes per lane (two to eight vectors)
     constexpr int NBr = 128 / (V * (int)sizeof(T));
     constexpr int NB = NBr < 2 ? 2 : (NBr > 8 ? 8 : NBr);
@@ -907,6 +907,65 @@ __global__ void __launch_bounds__(kThreads, MBL_TILED_MIN_BLOCKS) k_apply_tiled(
     }
     if (MODE == kPlain) return;
     pcg_block_finish<T, V, G, MODE>(red, part, K, ps, rd);
+}
+
+// Any block width: the tiled product with the width, and so the lanes of a row, known at run
+// time only.  A row takes G = k / V <= 16 lanes, a warp 32 / G rows at a time, and the lanes
+// left over repeat a row without storing it.  V elements a lane, as many as k, the leading
+// dimensions and the pointers allow (any_vector).  Against the kernel that gives a warp to
+// each row and ranks every neighbour (L = 20, k = 24, FP32): 77 -> 29 us.
+template <typename T, int V>
+__global__ void __launch_bounds__(kThreads, MBL_TILED_MIN_BLOCKS)
+    k_apply_any(ChainParams cp, int B, uint32_t CH, const T *__restrict__ X, int64_t ldx, T *__restrict__ Y, int64_t ldy, int k)
+{
+    constexpr int NBr = 128 / (V * (int)sizeof(T));
+    constexpr int NB = NBr < 2 ? 2 : (NBr > 8 ? 8 : NBr);
+    __shared__ uint32_t sbin[kBinomDim * kBinomDim];
+    __shared__ T tab[1024];
+    __shared__ uint32_t spref[kLowMaxB + 2];
+    __shared__ TileMeta<T> s_meta[kWarps];
+    load_binom(sbin);
+    build_field_tables<T>(tab, cp);
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        uint32_t acc = 0;
+        for (int q = 0; q <= B + 1 && q <= kLowMaxB + 1; ++q) {
+            spref[q] = acc;
+            acc += binom(sbin, B, q);
+        }
+    }
+    __syncthreads();
+    const int L = cp.L, m = cp.n_up, H = L - B;
+    const int G = k / V, RPW = 32 / G;
+    const uint32_t nchunk = (binom(sbin, B, B / 2) + CH - 1) / CH, total = (1u << H) * nchunk;
+    const T hdelta = cp_half_delta<T>(cp);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int grp = min(lane / G, RPW - 1), col = (lane % G) * V;
+    const bool spare = lane >= RPW * G;
+    const LowRec *__restrict__ tbl = g_lowtab + lowtab_base(B);
+    TileMeta<T> &tm = s_meta[warp];
+    T part[V];
+    for (uint32_t item = blockIdx.x * kWarps + warp; item < total; item += gridDim.x * kWarps) {
+        const uint32_t t = item / nchunk, c = item % nchunk;
+        const int p = m - __popc(t);
+        if (p < 0 || p > B) continue;  // warp-uniform
+        const uint32_t Rt = binom(sbin, B, p), j_begin = c * CH;
+        if (j_begin >= Rt) continue;
+        const uint32_t j_end = min(Rt, j_begin + CH);
+        __syncwarp();
+        tile_meta_warp<T>(sbin, tab, cp, B, t, p, tm);
+        __syncwarp();
+        const uint32_t t0 = t & 1u, thi = (t >> (H - 1)) & 1u;
+        const uint32_t sup = p >= 1 ? binom(sbin, B - 1, p - 1) : 0u, sdn = binom(sbin, B - 1, p);
+        const LowRec *__restrict__ rp = tbl + spref[p];
+        const T *__restrict__ Xt = X + (int64_t)tm.off * ldx;
+        for (uint32_t j0 = j_begin; j0 < j_end; j0 += RPW) {
+            const uint32_t j = j0 + grp;
+            tile_row_pass<T, V, NB, kPlain>(cp, B, X, ldx, Xt, ldx, rp, min(j, j_end - 1u), !spare && j < j_end, tm, tab,
+                                            hdelta, t0, thi, sup, sdn, col, Y, ldy, nullptr, nullptr, nullptr, part,
+                                            nullptr, nullptr);
+        }
+    }
 }
 
 // ---------------------------------------------------------------------------------
@@ -1864,7 +1923,22 @@ int ensure_lowtab(int B)
     return MBL_OK;
 }
 
-// Runtime block width (any 1 <= k <= 256, any alignment): one warp per row, lanes
+// Whether a product of tile width B can be enqueued on st now: the table is on the device, or
+// st is not being captured (its upload is a synchronous copy).
+static bool lowtab_usable(int B, cudaStream_t st)
+{
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return false;
+    {
+        std::lock_guard<std::mutex> lock(g_lowtab_mutex);
+        if (g_lowtab_ready[dev][B]) return true;
+    }
+    cudaStreamCaptureStatus status;
+    return cudaStreamIsCapturing(st, &status) == cudaSuccess && status == cudaStreamCaptureStatusNone;
+}
+
+// Untiled product (chains of fewer than four sites, tile bits -1, or a capture that meets a
+// tile width for the first time) of any block width and alignment: one warp per row, lanes
 // stride the columns.  Plain product only.
 template <typename T>
 __global__ void __launch_bounds__(kThreads) k_apply_generic(ChainParams cp, const T *__restrict__ X,
@@ -3117,6 +3191,18 @@ static int lane_bytes_for(int L, int K, size_t es)
     return size_lane_bytes(K, es);
 }
 
+// Rows per work item of the tiled kernels: `most`, or as few as still give every resident
+// warp an item when the sector is small, so that its rows are not passed over one after
+// another by a few warps (a pass is a chain of three dependent loads).  Measured on GB300
+// against always `most`: FP32 L = 12, k = 8 8.8 -> 5.3 us, L = 16, k = 16 11.1 -> 6.6 us; FP64
+// L = 14, k = 16 42 -> 16 us, L = 18, k = 32 90 -> 72 us.
+static uint32_t chunk_rows(uint32_t n, uint32_t rows_per_pass, int resident_warps, uint32_t most)
+{
+    const uint64_t pass = (uint64_t)rows_per_pass * (uint64_t)resident_warps;
+    const uint64_t rows = rows_per_pass * ((n + pass - 1) / pass);
+    return rows < most ? (uint32_t)rows : most;
+}
+
 template <typename T, int K, int MODE, int LB>
 static cudaError_t launch_tiled_lb(const ChainParams &cp, int B, const T *X, int64_t ldx, T *Y, int64_t ldy, T *R,
                                    const T *dinv, const PcgScalars &ps, const Reduce &rd, cudaStream_t st)
@@ -3130,17 +3216,19 @@ static cudaError_t launch_tiled_lb(const ChainParams &cp, int B, const T *X, int
         return v;
     }();
     const uint32_t rmax = host_binom(B, B / 2);
-    constexpr int CH = WideRowLayout<T, K, LB>::CH;
-    const int64_t items = ((int64_t)1 << (cp.L - B)) * (int64_t)((rmax + CH - 1) / CH);
     int64_t grid = (int64_t)num_sms() * per_sm;
     if (grid > (int64_t)num_sms() * 8) grid = (int64_t)num_sms() * 8;  // partials capacity
-    const int64_t need = (items + kWarps - 1) / kWarps;
     // the ordered schedule (one item per warp) only for the plain product: the PCG
     // epilogues keep one partial per block in a buffer sized for the persistent grid
-    if (MODE == kPlain && ordered_schedule(cp.L, cp.n_up, K, sizeof(T))) grid = need;
+    const bool ordered = MODE == kPlain && ordered_schedule(cp.L, cp.n_up, K, sizeof(T));
+    using Lay = WideRowLayout<T, K, LB>;
+    const uint32_t CH = ordered ? (uint32_t)Lay::CH
+                                : chunk_rows(host_binom(cp.L, cp.n_up), 32 / Lay::G, (int)grid * kWarps, Lay::CH);
+    const int64_t items = ((int64_t)1 << (cp.L - B)) * (int64_t)((rmax + CH - 1) / CH);
+    const int64_t need = (items + kWarps - 1) / kWarps;
+    if (ordered || grid > need) grid = need;
     note_launch();
-    if (grid > need) grid = need;
-    kern<<<(int)grid, kThreads, 0, st>>>(cp, B, X, ldx, Y, ldy, R, dinv, ps, rd);
+    kern<<<(int)grid, kThreads, 0, st>>>(cp, B, CH, X, ldx, Y, ldy, R, dinv, ps, rd);
     return cudaGetLastError();
 }
 
@@ -3346,6 +3434,66 @@ static bool vec_ok(const void *p, int64_t ld, int K)
     return ((uintptr_t)p % align == 0) && ((ld * (int64_t)sizeof(T)) % align == 0);
 }
 
+// Elements per lane of the any-width kernel: a divisor of the width, up to 32 bytes, that the
+// pointers and leading dimensions are aligned to.
+template <typename T>
+static int any_vector(const void *X, int64_t ldx, const void *Y, int64_t ldy, int k)
+{
+    for (int v = 32 / (int)sizeof(T); v > 1; v /= 2) {
+        const size_t b = (size_t)v * sizeof(T);
+        if (k % v == 0 && (uintptr_t)X % b == 0 && (uintptr_t)Y % b == 0 && (ldx * (int64_t)sizeof(T)) % (int64_t)b == 0 &&
+            (ldy * (int64_t)sizeof(T)) % (int64_t)b == 0)
+            return v;
+    }
+    return 1;
+}
+
+// The any-width kernel does a row's index work in each of its lanes: it pays where a warp
+// takes two rows or more at a time (FP32, L = 20: k = 24 77 -> 29 us; k = 32 with an odd
+// leading dimension, a row a pass, 139 against the row-a-warp kernel's 78 us).
+template <typename T>
+static bool any_width_ok(const void *X, int64_t ldx, const void *Y, int64_t ldy, int k)
+{
+    return k / any_vector<T>(X, ldx, Y, ldy, k) <= 16;
+}
+
+template <typename T, int V>
+static cudaError_t launch_any_v(const ChainParams &cp, int B, const T *X, int64_t ldx, T *Y, int64_t ldy, int k,
+                                cudaStream_t st)
+{
+    auto kern = k_apply_any<T, V>;
+    static const int per_sm = [&]() {
+        int v = 0;
+        cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, 25);
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, kern, kThreads, 0) != cudaSuccess || v < 1) v = 1;
+        return v;
+    }();
+    const int RPW = 32 / (k / V);
+    const int64_t cap = (int64_t)num_sms() * per_sm;
+    const uint32_t rmax = host_binom(B, B / 2);
+    const uint32_t CH = chunk_rows(host_binom(cp.L, cp.n_up), (uint32_t)RPW, (int)cap * kWarps,
+                                   (uint32_t)(MBL_CH_PASSES * RPW > 32 ? MBL_CH_PASSES * RPW : 32));
+    const int64_t items = ((int64_t)1 << (cp.L - B)) * (int64_t)((rmax + CH - 1) / CH);
+    const int64_t need = (items + kWarps - 1) / kWarps;
+    note_launch();
+    kern<<<(int)(need < cap ? need : cap), kThreads, 0, st>>>(cp, B, CH, X, ldx, Y, ldy, k);
+    return cudaGetLastError();
+}
+
+template <typename T>
+static cudaError_t launch_any(const ChainParams &cp, int B, const T *X, int64_t ldx, T *Y, int64_t ldy, int k,
+                              cudaStream_t st)
+{
+    if (ensure_lowtab(B) != MBL_OK) return cudaErrorUnknown;
+    switch (any_vector<T>(X, ldx, Y, ldy, k)) {
+    case 8:
+        if constexpr (sizeof(T) == 4) return launch_any_v<T, 8>(cp, B, X, ldx, Y, ldy, k, st);
+    case 4: return launch_any_v<T, 4>(cp, B, X, ldx, Y, ldy, k, st);
+    case 2: return launch_any_v<T, 2>(cp, B, X, ldx, Y, ldy, k, st);
+    default: return launch_any_v<T, 1>(cp, B, X, ldx, Y, ldy, k, st);
+    }
+}
+
 template <typename T>
 static int dispatch_plain(const ChainParams &cp, const T *X, int64_t ldx, T *Y, int64_t ldy, uint32_t n, int k,
                           cudaStream_t st)
@@ -3368,7 +3516,7 @@ static int dispatch_plain(const ChainParams &cp, const T *X, int64_t ldx, T *Y, 
         case 64: e = launch_tiled<T, 64, kPlain>(cp, B, X, ldx, Y, ldy, nullptr, nullptr, ps, rd, st); break;
         default: done = false;
         }
-    } else if (vec_ok<T>(X, ldx, k) && vec_ok<T>(Y, ldy, k)) {
+    } else if (B < 2 && vec_ok<T>(X, ldx, k) && vec_ok<T>(Y, ldy, k)) {
         switch (k) {
         case 1: e = launch_apply_k<T, 1, kPlain>(cp, X, ldx, Y, ldy, n, nullptr, nullptr, ps, rd, grid, st); break;
         case 2: e = launch_apply_k<T, 2, kPlain>(cp, X, ldx, Y, ldy, n, nullptr, nullptr, ps, rd, grid, st); break;
@@ -3382,7 +3530,9 @@ static int dispatch_plain(const ChainParams &cp, const T *X, int64_t ldx, T *Y, 
     } else {
         done = false;
     }
-    if (!done) {
+    if (!done && B >= 2 && any_width_ok<T>(X, ldx, Y, ldy, k) && lowtab_usable(B, st)) {
+        e = launch_any<T>(cp, B, X, ldx, Y, ldy, k, st);
+    } else if (!done) {
         const size_t sm = apply_smem_bytes<T>();
         static const bool attr_set_once = [&]() {
             cudaFuncSetAttribute(k_apply_generic<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
