@@ -16,8 +16,9 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
-#include <cmath>
+#include <algorithm>
 #include <atomic>
+#include <cmath>
 #include <mutex>
 #include <vector>
 
@@ -572,7 +573,7 @@ struct LowRec {
     uint8_t cnt;     // flippable bonds inside the low part
     uint8_t alow;    // antiparallel bonds inside the low part
     uint16_t jper;   // colex rank of u ^ 1 among the words of its popcount
-    uint16_t pad;
+    uint16_t j;      // colex rank of u itself
     uint16_t nb[12];  // in-tile ranks of the low-part neighbours
 };
 static_assert(sizeof(LowRec) == 32, "LowRec layout");
@@ -581,8 +582,24 @@ constexpr int kLowMaxB = 13;  // at most 12 low bonds, C(13, 6) = 1716 rows per 
 // records for B = 2..13 at offsets 2^B - 4 (the sizes 2^B, B < current, summed)
 constexpr int kLowRecords = (1 << (kLowMaxB + 1)) - 4;
 static __device__ __align__(16) LowRec g_lowtab[kLowRecords];
+// The same records, those of one popcount ordered by (neighbours, top bit, bottom bit): the
+// order in which FP64 products take the rows of a tile.  A warp's rows then have the same
+// in-tile neighbours to add, and a joining or wrap partner all or none of them; in rank order
+// the warp went through the largest of their counts, and an FP64 addition holds a quarter of
+// an SM's FP64 pipe for 64 cycles whichever lanes need it (L = 22, k = 32: 817 -> 760 us;
+// k = 12: 403 -> 375 us).
+static __device__ __align__(16) LowRec g_lowtab_f64[kLowRecords];
+
 
 __host__ __device__ inline int lowtab_base(int B) { return (1 << B) - 4; }
+
+// The table for blocks of k columns: rank order for FP32, and for FP64 rows below 64 bytes,
+// whose neighbours share memory sectors.
+template <typename T>
+__device__ __forceinline__ const LowRec *low_table(int B, int k)
+{
+    return (sizeof(T) == 8 && k >= 8 ? g_lowtab_f64 : g_lowtab) + lowtab_base(B);
+}
 
 // Resident blocks per SM the tiled kernel is compiled for (register budget 65536 /
 // (256 * this)); 3 keeps every variant free of spills.
@@ -683,9 +700,10 @@ __device__ __forceinline__ void half_sum_plus_dx(T (&acc)[V], const T (&nb)[V], 
     }
 }
 
-// One pass of a warp over RPW rows of a tile (row j of this lane group, `valid` when it
-// is a row of the work item; otherwise j is some other row of the same tile and only the
-// output is dropped).  Own row and in-tile neighbours come from Xt (row stride ldt: the
+// One pass of a warp over RPW rows of a tile (record i of the table for this lane group,
+// `valid` when it is a row of the work item; otherwise i is some other record of the same
+// tile and only the output is dropped); its row of the tile is i in FP32, record i's j in
+// FP64 (the tables of low_table differ in their order).  Own row and in-tile neighbours come from Xt (row stride ldt: the
 // tile in shared memory, or X itself from the tile's first row); the joining, wrap and
 // high-bond rows from X.  y = (d - sigma) x + 1/2 (sum of neighbour rows), the
 // neighbours summed first in a fixed order (low bonds, joining, wrap, high bonds):
@@ -699,7 +717,7 @@ __device__ __forceinline__ void half_sum_plus_dx(T (&acc)[V], const T (&nb)[V], 
 template <typename T, int V, int NB, int MODE>
 __device__ __forceinline__ void tile_row_pass(const ChainParams &cp, int B, const T *__restrict__ X, int64_t ldx,
                                               const T *__restrict__ Xt, int64_t ldt, const LowRec *__restrict__ rp,
-                                              uint32_t j, bool valid, const TileMeta<T> &tm, const T *tab, T hdelta,
+                                              uint32_t i, bool valid, const TileMeta<T> &tm, const T *tab, T hdelta,
                                               uint32_t t0, uint32_t thi, uint32_t sup, uint32_t sdn, int col,
                                               T *__restrict__ Y, int64_t ldy, T *__restrict__ R,
                                               const T *__restrict__ dinv, const T *s_alpha, T (&part)[V],
@@ -710,10 +728,11 @@ __device__ __forceinline__ void tile_row_pass(const ChainParams &cp, int B, cons
     constexpr int kEarly = MBL_ROW_EARLY_BYTES / kVecBytes - 2 > 0 ? MBL_ROW_EARLY_BYTES / kVecBytes - 2 : 0;
     // in-tile rows requested together (64 bytes per lane)
     constexpr int NBL = 64 / kVecBytes > 1 ? 64 / kVecBytes : 1;
+    const uint4 w0 = __ldg(reinterpret_cast<const uint4 *>(rp + i));
+    const uint4 w1 = __ldg(reinterpret_cast<const uint4 *>(rp + i) + 1);
+    const uint32_t j = sizeof(T) == 8 ? w0.y >> 16 : i;
     const uint32_t r = tm.off + j;
     const T *__restrict__ xr = X + (int64_t)r * ldx + col;
-    const uint4 w0 = __ldg(reinterpret_cast<const uint4 *>(rp + j));
-    const uint4 w1 = __ldg(reinterpret_cast<const uint4 *>(rp + j) + 1);
     const uint32_t u = w0.x & 0xffffu, cnt = (w0.x >> 16) & 0xffu, alow = w0.x >> 24;
     const uint32_t ub = (u >> (B - 1)) & 1u;
     const bool join = ub != t0;
@@ -874,7 +893,7 @@ __global__ void __launch_bounds__(kThreads, MBL_TILED_MIN_BLOCKS) k_apply_tiled(
     const T hdelta = cp_half_delta<T>(cp);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, grp = lane / G;
     const int col = (lane % G) * V;
-    const LowRec *__restrict__ tbl = g_lowtab + lowtab_base(B);
+    const LowRec *__restrict__ tbl = low_table<T>(B, K);
     TileMeta<T> &tm = s_meta[warp];
     T part[V];
 #pragma unroll
@@ -942,7 +961,7 @@ __global__ void __launch_bounds__(kThreads, MBL_TILED_MIN_BLOCKS)
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int grp = min(lane / G, RPW - 1), col = (lane % G) * V;
     const bool spare = lane >= RPW * G;
-    const LowRec *__restrict__ tbl = g_lowtab + lowtab_base(B);
+    const LowRec *__restrict__ tbl = low_table<T>(B, k);
     TileMeta<T> &tm = s_meta[warp];
     T part[V];
     for (uint32_t item = blockIdx.x * kWarps + warp; item < total; item += gridDim.x * kWarps) {
@@ -1069,7 +1088,7 @@ __global__ void __launch_bounds__(kThreads, MBL_STAGED_MIN_BLOCKS)
     const T hdelta = cp_half_delta<T>(cp);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, grp = lane / G;
     const int col = (lane % G) * V;
-    const LowRec *__restrict__ tbl = g_lowtab + lowtab_base(B);
+    const LowRec *__restrict__ tbl = low_table<T>(B, K);
     T part[V];
 #pragma unroll
     for (int v = 0; v < V; ++v) part[v] = (T)0;
@@ -1896,9 +1915,10 @@ int ensure_lowtab(int B)
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return MBL_ERR_CUDA;
     std::lock_guard<std::mutex> lock(g_lowtab_mutex);
     if (g_lowtab_ready[dev][B]) return MBL_OK;
-    std::vector<LowRec> recs((size_t)1 << B);
+    std::vector<LowRec> recs((size_t)1 << B), sorted;
     size_t idx = 0;
     for (int p = 0; p <= B; ++p) {
+        const size_t first = idx;
         // words of popcount p in ascending order: their position is their colex rank
         for (uint32_t u = 0; u < (1u << B); ++u) {
             if (__builtin_popcount(u) != p) continue;
@@ -1913,11 +1933,17 @@ int ensure_lowtab(int B)
             rec.cnt = (uint8_t)cnt;
             rec.alow = (uint8_t)cnt;
             rec.jper = (uint16_t)host_colex_rank(u ^ 1u);
+            rec.j = (uint16_t)(idx - first);
             recs[idx++] = rec;
         }
+        sorted.insert(sorted.end(), recs.begin() + (long)first, recs.begin() + (long)idx);
+        auto key = [B](const LowRec &r) { return (r.cnt << 2) | (((r.u >> (B - 1)) & 1) << 1) | (r.u & 1); };
+        std::stable_sort(sorted.begin() + (long)first, sorted.end(),
+                         [&](const LowRec &x, const LowRec &y) { return key(x) < key(y); });
     }
-    if (cudaMemcpyToSymbol(g_lowtab, recs.data(), recs.size() * sizeof(LowRec),
-                           (size_t)lowtab_base(B) * sizeof(LowRec)) != cudaSuccess)
+    const size_t bytes = recs.size() * sizeof(LowRec), at = (size_t)lowtab_base(B) * sizeof(LowRec);
+    if (cudaMemcpyToSymbol(g_lowtab, recs.data(), bytes, at) != cudaSuccess ||
+        cudaMemcpyToSymbol(g_lowtab_f64, sorted.data(), bytes, at) != cudaSuccess)
         return MBL_ERR_CUDA;
     g_lowtab_ready[dev][B] = true;
     return MBL_OK;
@@ -2480,7 +2506,7 @@ __device__ __noinline__ void run_product()
     T *Y = MODE != kPcgQ ? as_global<T>(Ln.t) : nullptr;
     T *R = MODE == kPcgQ ? as_global<T>(Ln.r) : nullptr;
     const T *dinv = as_global<T>(const_cast<void *>(Ln.dinv));
-    const LowRec *tbl = g_lowtab + lowtab_base(B);
+    const LowRec *tbl = low_table<T>(B, K);
     const RunShare sh = run_share<STAGED>(Ln);
     T part[V];
 #pragma unroll
