@@ -152,14 +152,21 @@ def _check(rc, what, ok=(MBL_OK,)):
     return rc
 
 
+@functools.lru_cache(maxsize=1)
 def _torch():
     import torch
     return torch
 
 
 def _stream_ptr(t):
+    """torch's current stream on the tensor's device.  Asked for as the raw handle where torch
+    has it (0.2 us; building a Stream object took 2.2 of the 9.3 us that a small product's call
+    takes on the host)."""
     torch = _torch()
-    return ctypes.c_void_p(torch.cuda.current_stream(t.device).cuda_stream)
+    raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+    if raw is None:
+        return ctypes.c_void_p(torch.cuda.current_stream(t.device).cuda_stream)
+    return ctypes.c_void_p(raw(t.device.index))
 
 
 def _dev(t, dtype, what):
