@@ -40,9 +40,62 @@ struct Eps<double> {
 // different bank in every lane.
 __host__ __device__ inline int pad_ld(int n) { return n | 1; }
 
+// The rotation (c, s) of one pair, or false where |a_pq| <= eps sqrt(|a_pp a_qq|):
+// t = sign(tau) / (|tau| + sqrt(1 + tau^2)), tau = (a_qq - a_pp) / (2 a_pq), c = 1 / sqrt(1 +
+// t^2), s = t c.
+template <typename T>
+__device__ __forceinline__ bool jacobi_rotation_exact(T apq, T app, T aqq, T &c, T &s)
+{
+    if (apq == (T)0 || !(fabs(apq) > Eps<T>::v() * sqrt(fabs(app * aqq)))) return false;
+    const T tau = (aqq - app) / ((T)2 * apq);
+    const T t = (tau >= (T)0 ? (T)1 : (T)-1) / (fabs(tau) + sqrt((T)1 + tau * tau));
+    c = (T)1 / sqrt((T)1 + t * t);
+    s = t * c;
+    return true;
+}
+
+__device__ __forceinline__ bool jacobi_rotation(float apq, float app, float aqq, float &c, float &s)
+{
+    return jacobi_rotation_exact<float>(apq, app, aqq, c, s);
+}
+
+// FP64: the two divisions and three roots of the above are some hundred instructions of 64
+// cycles each on GB300's FP64 pipe, more than the rest of a round.  A rotation only has to be
+// orthogonal to FP64; that it leaves a_pq at 1e-7 of its value instead of zero costs nothing,
+// the sweeps converge as before.  So t comes from FP32, from a_qq - a_pp and a_pq scaled by a
+// common power of two, and c = 1 / sqrt(1 + t^2) from an FP32 start and two Newton steps in
+// FP64 (relative error 1e-7 -> 1e-14 -> below rounding).  H Rayleigh-Ritz at k = 32, Grams
+// and updates included: 2.01 -> 1.77 ms at L = 20, 1.36 -> 1.13 ms at L = 18.
+__device__ __forceinline__ bool jacobi_rotation(double apq, double app, double aqq, double &c, double &s)
+{
+    if (apq == 0.0) return false;
+    if (!(apq * apq > (Eps<double>::v() * Eps<double>::v()) * fabs(app * aqq))) {
+        // below the bound, or squares that underflow (or overflow, or a NaN): the plain test
+        if (fabs(apq) > 1e-140) return false;
+        return jacobi_rotation_exact<double>(apq, app, aqq, c, s);
+    }
+    const double d = aqq - app;
+    const int hd = __double2hiint(d) & 0x7ff00000, ha = __double2hiint(apq) & 0x7ff00000;
+    const int e = max(hd, ha);
+    // exponents within 100 of each other, away from the ends of the range
+    if (ha < e - (100 << 20) || e < (200 << 20) || e > (1900 << 20))
+        return jacobi_rotation_exact<double>(apq, app, aqq, c, s);
+    const int shift = (1023 << 20) - e;
+    const float df = hd < e - (100 << 20) ? 0.0f : (float)__hiloint2double(__double2hiint(d) + shift, __double2loint(d));
+    const float af = (float)__hiloint2double(__double2hiint(apq) + shift, __double2loint(apq));
+    const float tau = df / (2.0f * af);
+    const float tf = copysignf(1.0f, tau) / (fabsf(tau) + sqrtf(fmaf(tau, tau, 1.0f)));
+    const double t = (double)tf, u = fma(t, t, 1.0);
+    double y = (double)rsqrtf((float)u);
+    y = y * fma(-0.5 * u, y * y, 1.5);
+    y = y * fma(-0.5 * u, y * y, 1.5);
+    c = y;
+    s = t * y;
+    return true;
+}
+
 // Parallel cyclic Jacobi on the symmetric n x n matrix A (row stride ld): the
-// round-robin (circle) ordering rotates n/2 disjoint pairs per round.  A rotation zeroes
-// a_pq with t = sign(tau)/(|tau| + sqrt(1 + tau^2)), tau = (a_qq - a_pp)/(2 a_pq); pairs
+// round-robin (circle) ordering rotates n/2 disjoint pairs per round (jacobi_rotation); pairs
 // with |a_pq| <= eps sqrt(|a_pp a_qq|) are skipped (the relative test keeps the small
 // eigenvalues of graded matrices accurate); sweeps stop when one rotates nothing or after
 // max_sweeps.  On exit diag(A) holds the eigenvalues and the columns of V (stride ld)
@@ -58,7 +111,6 @@ __device__ void dev_jacobi(int n, int ld, T *A, T *V, T *cs, int *pairs, int *s_
     if (n < 2) return;
     const int np = (n + 1) & ~1;
     const int half = np / 2;
-    const T eps = Eps<T>::v();
     for (int sweep = 0; sweep < max_sweeps; ++sweep) {
         if (tid == 0) *s_rot = 0;
         __syncthreads();
@@ -78,16 +130,7 @@ __device__ void dev_jacobi(int n, int ld, T *A, T *V, T *cs, int *pairs, int *s_
                     q = t;
                 }
                 T c = (T)1, s = (T)0;
-                if (q < n) {
-                    const T apq = A[p * ld + q], app = A[p * ld + p], aqq = A[q * ld + q];
-                    if (apq != (T)0 && fabs(apq) > eps * sqrt(fabs(app * aqq))) {
-                        const T tau = (aqq - app) / ((T)2 * apq);
-                        const T t = (tau >= (T)0 ? (T)1 : (T)-1) / (fabs(tau) + sqrt((T)1 + tau * tau));
-                        c = (T)1 / sqrt((T)1 + t * t);
-                        s = t * c;
-                        *s_rot = 1;
-                    }
-                }
+                if (q < n && jacobi_rotation(A[p * ld + q], A[p * ld + p], A[q * ld + q], c, s)) *s_rot = 1;
                 pairs[2 * i] = p;
                 pairs[2 * i + 1] = q;
                 cs[2 * i] = c;
