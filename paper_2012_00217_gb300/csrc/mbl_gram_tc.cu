@@ -105,7 +105,7 @@ __device__ __forceinline__ void mma_commit(uint64_t *m)
 //                operand buffers, deep enough to cover the MMA-to-commit round trip,
 //   warp 25      MMA issuer (one thread): two k-steps of three kind::tf32 MMAs per box into
 //                one of two tensor-memory accumulators,
-//   warp 26      C producer: the tile's C (q/16 boxes) into one of one or two C/D slots,
+//   warp 26      C producer: the tile's C (q/16 boxes) into one of up to four C/D slots,
 //   warps 0-7    epilogue: tcgen05.ld of the accumulator (warp w reads lanes 32 (w % 4) .. +31,
 //                thread = row, w / 4 picks alternate 16-column groups), D = beta C + alpha acc
 //                in FP32 (C rounded to FP32 like the other inputs; FP64 arithmetic here would be
@@ -124,11 +124,12 @@ constexpr int kUpdBoxBytes = 16384;    // 128 rows x 16 FP64 columns, one ring s
 constexpr int kUpdKC = 16;             // K columns per ring slot
 constexpr int kUpdOpBytes = 8192;      // one TF32 operand part of a slot: 128 rows x 16 K
 constexpr int kUpdMaxStages = 8;
+constexpr int kUpdMaxC = 4;            // at most this many C/D slots
 constexpr int kUpdSmemMax = 230400;    // dynamic shared memory asked for (227 KB less the static part)
 
 struct UpdBars {
     uint64_t full[kUpdMaxStages], empty[kUpdMaxStages];
-    uint64_t afull[kUpdOpBufs], aempty[kUpdOpBufs], accfull[2], accempty[2], cfull[2], cempty[2], done;
+    uint64_t afull[kUpdOpBufs], aempty[kUpdOpBufs], accfull[2], accempty[2], cfull[kUpdMaxC], cempty[kUpdMaxC], done;
 };
 
 __device__ __forceinline__ void mbar_arrive1(uint64_t *m)
@@ -319,7 +320,7 @@ __global__ void __launch_bounds__(kUpdThreads, 1)
             mbar_init(&bars.accfull[b], 1);
             mbar_init(&bars.accempty[b], kUpdEpiThreads);
         }
-        for (int b = 0; b < 2; ++b) {
+        for (int b = 0; b < ncs; ++b) {
             mbar_init(&bars.cfull[b], 1);
             mbar_init(&bars.cempty[b], 1);
         }
@@ -522,11 +523,11 @@ __global__ void __launch_bounds__(kUpdThreads, 1)
                 for (int bxi = 0; bxi < ncb; ++bxi)
                     tma_store_box(&tmD, 16 * bxi, y, saddr(tslot + (size_t)bxi * kUpdBoxBytes));
                 asm volatile("cp.async.bulk.commit_group;" ::: "memory");
-                // a slot is handed back once its store has read it: with two slots the previous
-                // tile's store, with one this tile's
-                if (ncs == 2) {
+                // a slot is handed back once its store has read it: with two slots or more the
+                // previous tile's store, with one this tile's
+                if (ncs >= 2) {
                     asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
-                    if (i >= 1) mbar_arrive1(&bars.cempty[(i - 1) % 2]);
+                    if (i >= 1) mbar_arrive1(&bars.cempty[(i - 1) % ncs]);
                 } else {
                     asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
                     mbar_arrive1(&bars.cempty[0]);
@@ -883,12 +884,16 @@ struct UpdConfig {
     int ncs, nab, ns;  // C/D slots, operand buffers, A ring slots (0: does not fit)
 };
 
-// the deepest buffering that fits: two C/D slots and four operand buffers with an A ring of
-// at least four slots, else one C/D slot, else two operand buffers (an A ring of two slots
-// already keeps the loads ahead; the operand buffers cover the MMA round trip)
+// the deepest buffering that fits.  Three C/D slots and two operand buffers come first: a
+// slot's round (C arrives, the epilogue rewrites it, D's store reads it) is the longest chain
+// at small p, and with two of them it set the pace (n = 184,756, C given: p = q = 32 43.8 ->
+// 37.3 us, p = 64 50.0 -> 45.4; n = 705,432, p = q = 32 138 -> 114 us; a fourth slot adds
+// nothing).  Then two C/D slots and four operand buffers with an A ring of at least four
+// slots, else one C/D slot, else two operand buffers (an A ring of two slots already keeps the
+// loads ahead; the operand buffers cover the MMA round trip).
 UpdConfig update_config(int p, int q)
 {
-    const int cfg[3][3] = {{2, 4, 4}, {1, 4, 2}, {1, 2, 2}};
+    const int cfg[4][3] = {{3, 2, 4}, {2, 4, 4}, {1, 4, 2}, {1, 2, 2}};
     for (const auto &c : cfg) {
         const size_t fixed = update_fixed_smem(p, q, c[0], c[1]);
         if (fixed >= (size_t)kUpdSmemMax) continue;
