@@ -3194,31 +3194,58 @@ static thread_local int t_force_schedule = 0, t_force_lane = 0;
 // warp striding over the (tile, chunk) items.  Ordered: one item per warp and as many
 // blocks as needed, so the hardware hands out blocks in index order and the tiles in
 // flight stay a narrow, advancing window; with the grid-stride loop, warps that meet
-// many empty chunks run ahead and the window widens beyond L2.  Every block of the
-// ordered grid repeats the shared-memory setup, so it only pays for wide rows: measured
-// on GB300, ordered wins for rows of >= 256 bytes once the block vector is >= 1 GiB
-// (FP32), or >= 128 MiB in FP64 (ALU-bound there), and loses elsewhere.
-// The staged schedule (whole tiles in shared memory) is the default for 128-byte rows
-// once the block vector outgrows 16 MB (measured: 2-6 % faster there, slower for
-// narrower and wider rows); anything else defaults to persistent.
+// many empty chunks run ahead and the window widens beyond L2.  Staged: whole tiles in
+// shared memory.  Measured on GB300 (us, persistent / ordered / staged):
+//   FP32 k = 16: L = 20 20.5 / 20.6 / 21.7;  L = 22 57 / 63 / 54;  L = 25 425 / 457 / 387
+//        k = 32: L = 19 18.5 / 18.5 / 20.5;  L = 22 100 / 113 / 93;  L = 25 901 / 868 / 755
+//        k = 64: L = 20 49.9 / 53.5 / 49.7;  L = 22 191 / 195 / 176;  L = 24 926 / 774 / 776;
+//                L = 25 1967 / 1548 / 1639
+//   FP64 k = 16: L = 20 131 / 131 / 127;  L = 22 435 / 410 / 440;  L = 25 3194 / 2996 / 3473
+//        k = 32: L = 18 69 / 88 / 78;  L = 20 231 / 213 / 223;  L = 22 842 / 762 / 837
+//        k = 64: L = 18 123 / 164 / 125;  L = 20 443 / 405 / 422;  L = 23 3088 / 2817 / 3296
+// so FP32 rows of 64 to 256 bytes are staged from 16 MB (256 bytes: 32 MB) and ordered from
+// 1 GiB (256 bytes and wider); FP64 rows of 128 bytes and more are ordered from 32 MB, those
+// of exactly 128 bytes staged from 16 MB to there.
 static int size_schedule(int L, int n_up, int K, size_t es)
 {
-    const double bytes = (double)host_binom(L, n_up) * K * (double)es;
-    if (K * (int)es >= 256 && bytes >= (es == 8 ? 128.0 * (1 << 20) : 1024.0 * (1 << 20))) return 2;
-    if (K * (int)es == 128 && bytes >= 16.0 * (1 << 20)) return 3;
-    return 1;
+    const double mb = (double)host_binom(L, n_up) * K * (double)es / (1 << 20);
+    const int row = K * (int)es;
+    if (es == 8) {
+        if (row >= 128 && mb >= 32.0) return 2;
+        return row == 128 && mb >= 16.0 ? 3 : 1;
+    }
+    if (row >= 256 && mb >= 1024.0) return 2;
+    return row >= 64 && row <= 256 && mb >= (row == 256 ? 32.0 : 16.0) ? 3 : 1;
 }
+
+static int explicit_schedule(int K, size_t es) { return g_schedule[es == 8 ? 1 : 0][kslot(K)]; }
 
 static int schedule_for(int L, int n_up, int K, size_t es)
 {
     if (t_force_schedule) return t_force_schedule;
-    const int o = g_schedule[es == 8 ? 1 : 0][kslot(K)];
+    const int o = explicit_schedule(K, es);
     if (o) return o;
     const int a = (L >= 0 && L <= kMaxL) ? g_tuned[es == 8 ? 1 : 0][kslot(K)][L].schedule : 0;
     if (a) return a;
     return size_schedule(L, n_up, K, es);
 }
-static bool ordered_schedule(int L, int n_up, int K, size_t es) { return schedule_for(L, n_up, K, es) == 2; }
+
+// Work order of the PCG launches (the vectors exceed L2 there): staged for rows of 128 bytes
+// and more.  us a step, persistent / staged: FP32 L = 22, k = 32 343 / 297, k = 64 683 / 563,
+// L = 24, k = 64 2903 / 2365; FP64 L = 20, k = 32 596 / 567.
+static int pcg_schedule(int L, int n_up, int K, size_t es)
+{
+    const int o = explicit_schedule(K, es);
+    if (o) return o;
+    return K * (int)es >= 128 && (double)host_binom(L, n_up) * K * (double)es >= 16.0 * (1 << 20) ? 3 : 1;
+}
+
+template <int MODE>
+static int launch_schedule(int L, int n_up, int K, size_t es)
+{
+    return MODE == kPlain ? schedule_for(L, n_up, K, es) : pcg_schedule(L, n_up, K, es);
+}
+
 
 // 32-byte lanes by default; 64-byte lanes for FP64 rows of >= 128 bytes (measured 13 %
 // faster: the FP64 products are ALU-bound and wider lanes repeat less index work).
@@ -3263,7 +3290,7 @@ static cudaError_t launch_tiled_lb(const ChainParams &cp, int B, const T *X, int
     if (grid > (int64_t)num_sms() * 8) grid = (int64_t)num_sms() * 8;  // partials capacity
     // the ordered schedule (one item per warp) only for the plain product: the PCG
     // epilogues keep one partial per block in a buffer sized for the persistent grid
-    const bool ordered = MODE == kPlain && ordered_schedule(cp.L, cp.n_up, K, sizeof(T));
+    const bool ordered = MODE == kPlain && schedule_for(cp.L, cp.n_up, K, sizeof(T)) == 2;
     using Lay = WideRowLayout<T, K, LB>;
     const uint32_t CH = ordered ? (uint32_t)Lay::CH
                                 : chunk_rows(host_binom(cp.L, cp.n_up), 32 / Lay::G, (int)grid * kWarps, Lay::CH);
@@ -3283,8 +3310,6 @@ static int staged_bits(int L, int K, size_t es)
     while (B >= 2 && (size_t)host_binom(B, B / 2) * K * es > (size_t)kStageBytes) --B;
     return B;
 }
-
-static bool staged_schedule(int L, int n_up, int K, size_t es) { return schedule_for(L, n_up, K, es) == 3; }
 
 template <typename T, int K, int MODE, int LB>
 static cudaError_t launch_staged_lb(const ChainParams &cp, int Bs, const T *X, T *Y, T *R, const T *dinv,
@@ -3308,8 +3333,6 @@ static cudaError_t launch_staged_lb(const ChainParams &cp, int Bs, const T *X, T
     kern<<<(int)grid, kThreads, dyn, st>>>(cp, Bs, X, Y, R, dinv, ps, rd);
     return cudaGetLastError();
 }
-
-static bool streamed_schedule(int L, int n_up, int K, size_t es) { return schedule_for(L, n_up, K, es) == 4; }
 
 // Dynamic shared memory a streamed block can have next to the kernel's static arrays.
 template <typename T, int K, int MODE>
@@ -3380,8 +3403,6 @@ static cudaError_t launch_streamed(const ChainParams &cp, int Bs, const T *X, T 
     return cudaGetLastError();
 }
 
-static bool slab_schedule(int L, int n_up, int K, size_t es) { return schedule_for(L, n_up, K, es) == 5; }
-
 // Tile width of the slab kernel: the widest table-backed B (<= L - 2) whose largest tile
 // fits one 32 KB ring slot (the consumers cover exactly that many rows).
 static int slab_bits(int L, int K, size_t es)
@@ -3414,11 +3435,12 @@ template <typename T, int K, int MODE>
 static cudaError_t launch_tiled(const ChainParams &cp, int B, const T *X, int64_t ldx, T *Y, int64_t ldy, T *R,
                                 const T *dinv, const PcgScalars &ps, const Reduce &rd, cudaStream_t st)
 {
+    const int order = launch_schedule<MODE>(cp.L, cp.n_up, K, sizeof(T));
     if constexpr (SlabLayout<T, K>::ok) {
         // slab: contiguous rows (ld = K), 16-byte aligned bases for the bulk copies; the
         // q-launch variant leaves w to the direction update
         auto al = [](const void *q) { return q == nullptr || (uintptr_t)q % 16 == 0; };
-        if (slab_schedule(cp.L, cp.n_up, K, sizeof(T)) && ldx == K && (Y == nullptr || ldy == K) && al(X) &&
+        if (order == 5 && ldx == K && (Y == nullptr || ldy == K) && al(X) &&
             al(Y) && al(R) && (MODE != kPcgQ || ps.w == nullptr)) {
             const int Bs = slab_bits(cp.L, K, sizeof(T));
             if (Bs >= 2) return launch_slab<T, K, MODE>(cp, Bs, X, Y, R, dinv, ps, rd, st);
@@ -3427,7 +3449,7 @@ static cudaError_t launch_tiled(const ChainParams &cp, int B, const T *X, int64_
     if constexpr (StreamLayout<T, K>::ok) {
         // streamed: contiguous rows (ld = K) and 16-byte aligned bases for every streamed block
         auto al = [](const void *q) { return q == nullptr || (uintptr_t)q % 16 == 0; };
-        if (streamed_schedule(cp.L, cp.n_up, K, sizeof(T)) && ldx == K && (Y == nullptr || ldy == K) && al(X) &&
+        if (order == 4 && ldx == K && (Y == nullptr || ldy == K) && al(X) &&
             al(Y) && al(R) && al(ps.w) && al(ps.p)) {
             const int Bs = stream_bits<T, K>(cp.L);
             if (Bs >= 2) return launch_streamed<T, K, MODE>(cp, Bs, X, Y, R, dinv, ps, rd, st);
@@ -3437,7 +3459,7 @@ static cudaError_t launch_tiled(const ChainParams &cp, int B, const T *X, int64_
         // staged: contiguous rows (ld = K) and 16-byte aligned bases for the bulk copies
         const bool aligned = ((uintptr_t)X % 16 == 0) && (Y == nullptr || (uintptr_t)Y % 16 == 0) &&
                              (R == nullptr || (uintptr_t)R % 16 == 0);
-        if (staged_schedule(cp.L, cp.n_up, K, sizeof(T)) && ldx == K && (Y == nullptr || ldy == K) && aligned) {
+        if (order == 3 && ldx == K && (Y == nullptr || ldy == K) && aligned) {
             const int Bs = staged_bits(cp.L, K, sizeof(T));
             if (Bs >= 2) {
                 const int lbs = lane_bytes_for(cp.L, K, sizeof(T));
@@ -3654,10 +3676,15 @@ static uint32_t run_rows_per_pass(int K, size_t es)
     return 32u / (uint32_t)(row >= lb ? row / lb : 1);
 }
 
-// How the products of a lane are split, from its sizes alone.
+// Whether a lane's products take whole tiles through shared memory: rows of 128 bytes from
+// 16 MB, unless the switch or the autotuner says otherwise (L = 18, k = 64: 48.9 us a step in
+// chunks, 50.0 staged; FP64 301 and 316; L = 20, k = 32: 87 and 82).
 static bool run_staged(int L, int n_up, int K, size_t es)
 {
-    return (K * (int)es) % 16 == 0 && schedule_for(L, n_up, K, es) == 3;
+    const int o = explicit_schedule(K, es), a = g_tuned[es == 8 ? 1 : 0][kslot(K)][L].schedule;
+    if ((K * (int)es) % 16 != 0) return false;
+    if (o || a) return (o ? o : a) == 3;
+    return K * (int)es == 128 && (double)host_binom(L, n_up) * K * (double)es >= 16.0 * (1 << 20);
 }
 
 static int run_staged_bits(int L, int K, size_t es)
