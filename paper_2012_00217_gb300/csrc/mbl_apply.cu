@@ -2201,13 +2201,13 @@ __global__ void __launch_bounds__(kThreads) k_pcg_update(uint32_t n, const T *__
 // through that order there and back (staged), or cut into row chunks dealt out to the warps.
 // Every block sums all partials of its lane itself, in a fixed order, right after the
 // barrier.  Measured (GB300, us a step, three launches -> resident):
-//   FP32  L = 12, k = 8: 32.8 -> 13.9;  14, 16: 35.9 -> 15.7;  16, 16: 40.3 -> 16.9;
-//         16, 64: 60.5 -> 22.3;  18, 32: 53.1 -> 31.0;  20, 32: 97.4 -> 83.8
-//   FP64  L = 14, k = 16: 118 -> 44.7;  18, 32: 236 -> 169
-// At L = 20, k = 32 the phases take about 22, 27 and 13 us of L2 traffic and the three
-// barriers with their sums the rest.  Beyond L2 (a lane's four vectors above 100 MB) the
-// launches are as fast or faster (L = 20, k = 64: 185 against 190 us; L = 22, k = 32: 301
-// against 404 us) and stay.
+//   FP32  L = 12, k = 8: 32.8 -> 13.9;  16, 16: 40.3 -> 16.4;  18, 32: 53.1 -> 29.3;
+//         20, 32: 97.4 -> 77.5
+//   FP64  L = 14, k = 16: 118 -> 44;  18, 32: 236 -> 164
+// At L = 20, k = 32 the phases take about 22, 27 and 11 us, bound by L2 gathers and streams
+// at the loads a block has in flight, and the three barriers with their sums the rest.
+// Beyond L2 (a lane's four vectors above 100 MB) the launches are as fast or faster (L = 20,
+// k = 64: 185 against 190 us; L = 22, k = 32: 301 against 404 us) and stay.
 //
 // A lane's blocks wait for one another, so the launch is cooperative.  Every wait is
 // bounded; on a time-out the lane's fail word is set, its blocks leave, and each writes
@@ -2383,7 +2383,7 @@ __device__ __forceinline__ bool lane_barrier(RunShared<T> &sm, unsigned &target)
 // column over the blocks.  In FP32 neither they nor the scalars that follow touch the FP64
 // pipe, where one warp's instruction takes 64 cycles however few of its lanes are active.
 template <typename T, int K, bool ASYNC>
-__device__ __forceinline__ bool lane_column_sums(double *buf, unsigned &target)
+__device__ __noinline__ bool lane_column_sums(double *buf, unsigned &target)
 {
     RunShared<T> &sm = run_shared<T>();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -2659,14 +2659,15 @@ __device__ __forceinline__ void run_move_w(uint32_t row_b, uint32_t row_e, uint3
 
 // w += alpha p, p = M^-1 r + beta p for rows [row_b, row_e), the block's share.  W_TMEM: w
 // stays in tensor memory for the whole launch, which takes two of the phase's five vector
-// streams off L2 (L = 20, k = 32: 25 -> 18 us for this phase; then three rows a thread in
-// flight instead of five, which spilled, 18 -> 13 us).
-constexpr int kRunUpdRows = 3;
+// streams off L2 (L = 20, k = 32: 25 -> 18 us for this phase).  A row a thread at a time and
+// inlined: more rows in flight cost more in saved and spilled registers than they gave (a
+// step at L = 20, k = 32: 91 us with seven rows, 82.4 with three, 78.8 with one, and 77.5
+// with the sums a function of their own instead).
 template <typename T, int K, bool W_TMEM>
-__device__ __noinline__ void run_update(uint32_t row_b, uint32_t row_e, uint32_t tmem)
+__device__ __forceinline__ void run_update(uint32_t row_b, uint32_t row_e, uint32_t tmem)
 {
     using Rows = RunRows<T, K>;
-    constexpr int V = Rows::V, G = Rows::G, RPP = Rows::RPP, U = kRunUpdRows;
+    constexpr int V = Rows::V, G = Rows::G, RPP = Rows::RPP;
     RunShared<T> &sm = run_shared<T>();
     const int col = (threadIdx.x % G) * V;
     T a[V], bt[V];
@@ -2677,52 +2678,45 @@ __device__ __noinline__ void run_update(uint32_t row_b, uint32_t row_e, uint32_t
     }
     const uint32_t slots = (row_e - row_b + RPP - 1) / RPP;
     uint32_t row = row_b + threadIdx.x / G;
-    // the thread's rows lie RPP apart: constant offsets from these pointers
     const int64_t at0 = (int64_t)row * K + col;
     const T *r = as_global<T>(sm.lane.r) + at0, *dinv = as_global<T>(const_cast<void *>(sm.lane.dinv)) + row;
     T *p = as_global<T>(sm.lane.p) + at0, *w = as_global<T>(sm.lane.w) + at0;
     constexpr int STEP = RPP * K;
     uint32_t slot = W_TMEM ? run_tmem_slot(tmem, 0) : 0u;
 #pragma unroll 1
-    for (uint32_t s0 = 0; s0 < slots; s0 += U) {
-        Vec<T, V> rv[U], pv[U];
-        T di[U];
-#pragma unroll
-        for (int q = 0; q < U; ++q)
-            if (row + q * RPP < row_e) {
-                rv[q] = ldv<T, V>(r + q * STEP);
-                pv[q] = ldv<T, V>(p + q * STEP);
-                di[q] = dinv[q * RPP];
-            }
-#pragma unroll
-        for (int q = 0; q < U; ++q) {
-            if (s0 + q >= slots) break;
-            const bool in = row + q * RPP < row_e;
-            if (W_TMEM) {
-                uint4 raw = tmem_ld4(slot + 4 * q);
-                Vec<T, V> wv = *reinterpret_cast<Vec<T, V> *>(&raw);
-#pragma unroll
-                for (int v = 0; v < V; ++v) wv.v[v] += a[v] * (in ? pv[q].v[v] : (T)0);
-                tmem_st4(slot + 4 * q, *reinterpret_cast<uint4 *>(&wv));
-            } else if (in) {
-                Vec<T, V> wv = ldv<T, V>(w + q * STEP);
-#pragma unroll
-                for (int v = 0; v < V; ++v) wv.v[v] += a[v] * pv[q].v[v];
-                stv<T, V>(w + q * STEP, wv);
-            }
-            if (in) {
-                Vec<T, V> pn;
-#pragma unroll
-                for (int v = 0; v < V; ++v) pn.v[v] = di[q] * rv[q].v[v] + bt[v] * pv[q].v[v];
-                stv<T, V>(p + q * STEP, pn);
-            }
+    for (uint32_t s = 0; s < slots; ++s) {  // the same for all threads: tcgen05 wants whole warps
+        const bool in = row < row_e;
+        Vec<T, V> rv, pv, wv;
+        T di = (T)0;
+        if (in) {
+            rv = ldv<T, V>(r);
+            pv = ldv<T, V>(p);
+            di = *dinv;
+            if (!W_TMEM) wv = ldv<T, V>(w);
         }
-        row += U * RPP;
-        r += U * STEP;
-        p += U * STEP;
-        w += U * STEP;
-        dinv += U * RPP;
-        slot += 4 * U;
+        if (W_TMEM) {
+            uint4 raw = tmem_ld4(slot);
+            wv = *reinterpret_cast<Vec<T, V> *>(&raw);
+#pragma unroll
+            for (int v = 0; v < V; ++v) wv.v[v] += a[v] * (in ? pv.v[v] : (T)0);
+            tmem_st4(slot, *reinterpret_cast<uint4 *>(&wv));
+        } else if (in) {
+#pragma unroll
+            for (int v = 0; v < V; ++v) wv.v[v] += a[v] * pv.v[v];
+            stv<T, V>(w, wv);
+        }
+        if (in) {
+            Vec<T, V> pn;
+#pragma unroll
+            for (int v = 0; v < V; ++v) pn.v[v] = di * rv.v[v] + bt[v] * pv.v[v];
+            stv<T, V>(p, pn);
+        }
+        row += RPP;
+        r += STEP;
+        p += STEP;
+        w += STEP;
+        dinv += RPP;
+        slot += 4;
     }
     if (W_TMEM) tmem_wait_st();
 }
