@@ -836,8 +836,10 @@ __device__ __forceinline__ void tile_row_pass(const ChainParams &cp, int B, cons
     }
 }
 
-template <typename T, int K, int MODE, int LB>
-__global__ void __launch_bounds__(kThreads, MBL_TILED_MIN_BLOCKS) k_apply_tiled(ChainParams cp, int B, uint32_t CH,
+// FULL: items of Lay::CH rows, a constant of the kernel (as a variable it cost the largest
+// products 0.6 %), else of ch.
+template <typename T, int K, int MODE, int LB, bool FULL>
+__global__ void __launch_bounds__(kThreads, MBL_TILED_MIN_BLOCKS) k_apply_tiled(ChainParams cp, int B, uint32_t ch,
                                                                                const T *__restrict__ X, int64_t ldx,
                                                                                T *__restrict__ Y, int64_t ldy,
                                                                                T *__restrict__ R,
@@ -846,6 +848,7 @@ __global__ void __launch_bounds__(kThreads, MBL_TILED_MIN_BLOCKS) k_apply_tiled(
 {
     using Lay = WideRowLayout<T, K, LB>;
     constexpr int V = Lay::V, G = Lay::G, RPW = 32 / G;
+    const uint32_t CH = FULL ? (uint32_t)Lay::CH : ch;
     // neighbour loads issued together: 128 bytes per lane (two to eight vectors)
     constexpr int NBr = 128 / (V * (int)sizeof(T));
     constexpr int NB = NBr < 2 ? 2 : (NBr > 8 ? 8 : NBr);
@@ -3267,32 +3270,47 @@ static uint32_t chunk_rows(uint32_t n, uint32_t rows_per_pass, int resident_warp
     return rows < most ? (uint32_t)rows : most;
 }
 
+// per_sm: resident blocks per SM of the kernel, with its preferred L1 share set.
+template <typename T, int K, int MODE, int LB, bool FULL>
+static int tiled_blocks_per_sm()
+{
+    static const int per_sm = []() {
+        auto kern = k_apply_tiled<T, K, MODE, LB, FULL>;
+        int v = 0;
+        cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, 25);
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, kern, kThreads, 0) != cudaSuccess || v < 1) v = 1;
+        return v > 8 ? 8 : v;  // partials capacity
+    }();
+    return per_sm;
+}
+
 template <typename T, int K, int MODE, int LB>
 static cudaError_t launch_tiled_lb(const ChainParams &cp, int B, const T *X, int64_t ldx, T *Y, int64_t ldy, T *R,
                                    const T *dinv, const PcgScalars &ps, const Reduce &rd, cudaStream_t st)
 {
     if (ensure_lowtab(B) != MBL_OK) return cudaErrorUnknown;
-    auto kern = k_apply_tiled<T, K, MODE, LB>;
-    static const int per_sm = [&]() {
-        int v = 0;
-        cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, 25);
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, kern, kThreads, 0) != cudaSuccess || v < 1) v = 1;
-        return v;
-    }();
-    const uint32_t rmax = host_binom(B, B / 2);
-    int64_t grid = (int64_t)num_sms() * per_sm;
-    if (grid > (int64_t)num_sms() * 8) grid = (int64_t)num_sms() * 8;  // partials capacity
+    using Lay = WideRowLayout<T, K, LB>;
     // the ordered schedule (one item per warp) only for the plain product: the PCG
     // epilogues keep one partial per block in a buffer sized for the persistent grid
     const bool ordered = MODE == kPlain && schedule_for(cp.L, cp.n_up, K, sizeof(T)) == 2;
-    using Lay = WideRowLayout<T, K, LB>;
-    const uint32_t CH = ordered ? (uint32_t)Lay::CH
-                                : chunk_rows(host_binom(cp.L, cp.n_up), 32 / Lay::G, (int)grid * kWarps, Lay::CH);
-    const int64_t items = ((int64_t)1 << (cp.L - B)) * (int64_t)((rmax + CH - 1) / CH);
+    int64_t grid = (int64_t)num_sms() * tiled_blocks_per_sm<T, K, MODE, LB, true>();
+    const uint32_t CH = ordered || MODE != kPlain
+                            ? (uint32_t)Lay::CH
+                            : chunk_rows(host_binom(cp.L, cp.n_up), 32 / Lay::G, (int)grid * kWarps, Lay::CH);
+    const bool full = CH == (uint32_t)Lay::CH;
+    if constexpr (MODE == kPlain)
+        if (!full) grid = (int64_t)num_sms() * tiled_blocks_per_sm<T, K, MODE, LB, false>();
+    const int64_t items = ((int64_t)1 << (cp.L - B)) * (int64_t)((host_binom(B, B / 2) + CH - 1) / CH);
     const int64_t need = (items + kWarps - 1) / kWarps;
     if (ordered || grid > need) grid = need;
     note_launch();
-    kern<<<(int)grid, kThreads, 0, st>>>(cp, B, CH, X, ldx, Y, ldy, R, dinv, ps, rd);
+    if constexpr (MODE == kPlain)
+        if (!full) {
+            k_apply_tiled<T, K, MODE, LB, false><<<(int)grid, kThreads, 0, st>>>(cp, B, CH, X, ldx, Y, ldy, R, dinv, ps,
+                                                                                 rd);
+            return cudaGetLastError();
+        }
+    k_apply_tiled<T, K, MODE, LB, true><<<(int)grid, kThreads, 0, st>>>(cp, B, CH, X, ldx, Y, ldy, R, dinv, ps, rd);
     return cudaGetLastError();
 }
 
