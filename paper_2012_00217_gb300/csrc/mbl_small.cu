@@ -66,6 +66,11 @@ __device__ __forceinline__ bool jacobi_rotation(float apq, float app, float aqq,
 // common power of two, and c = 1 / sqrt(1 + t^2) from an FP32 start and two Newton steps in
 // FP64 (relative error 1e-7 -> 1e-14 -> below rounding).  H Rayleigh-Ritz at k = 32, Grams
 // and updates included: 2.01 -> 1.77 ms at L = 20, 1.36 -> 1.13 ms at L = 18.
+// tau^2 has to stay within FP32: from |tau| = 2^64 on it overflows, t would be zero, and a pair
+// counted as rotated but left as it was keeps the sweeps going to their limit.  So pairs whose
+// a_qq - a_pp is 2^60 times a_pq and more (graded matrices) take the FP64 rotation.
+constexpr int kTauExponents = 60 << 20;  // in the high word of a double
+
 __device__ __forceinline__ bool jacobi_rotation(double apq, double app, double aqq, double &c, double &s)
 {
     if (apq == 0.0) return false;
@@ -77,11 +82,12 @@ __device__ __forceinline__ bool jacobi_rotation(double apq, double app, double a
     const double d = aqq - app;
     const int hd = __double2hiint(d) & 0x7ff00000, ha = __double2hiint(apq) & 0x7ff00000;
     const int e = max(hd, ha);
-    // exponents within 100 of each other, away from the ends of the range
-    if (ha < e - (100 << 20) || e < (200 << 20) || e > (1900 << 20))
+    // a_pq's exponent not far below the difference's, both away from the ends of the range (a
+    // difference far below a_pq is as good as zero: t is +-1 to FP64)
+    if (ha < e - kTauExponents || e < (200 << 20) || e > (1900 << 20))
         return jacobi_rotation_exact<double>(apq, app, aqq, c, s);
     const int shift = (1023 << 20) - e;
-    const float df = hd < e - (100 << 20) ? 0.0f : (float)__hiloint2double(__double2hiint(d) + shift, __double2loint(d));
+    const float df = hd < e - kTauExponents ? 0.0f : (float)__hiloint2double(__double2hiint(d) + shift, __double2loint(d));
     const float af = (float)__hiloint2double(__double2hiint(apq) + shift, __double2loint(apq));
     const float tau = df / (2.0f * af);
     const float tf = copysignf(1.0f, tau) / (fabsf(tau) + sqrtf(fmaf(tau, tau, 1.0f)));

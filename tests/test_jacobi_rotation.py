@@ -29,3 +29,28 @@ def test_rotation_is_orthogonal_and_annihilates(spread):
     left = (c * c - s * s) * apq + c * s * (app - aqq)
     # t is right to a few FP32 roundings: a_pq's share and the rotated diagonal's
     assert np.all(np.abs(left) <= 1e-6 * np.abs(apq) + 4e-16 * (np.abs(app) + np.abs(aqq)))
+
+
+def _guarded(apq, app, aqq):
+    """The rotation with its choice: beyond a difference of 2^60 times a_pq the FP64 formula."""
+    d = aqq - app
+    wide = np.frexp(d)[1] - np.frexp(apq)[1] > 60
+    with np.errstate(over="ignore", invalid="ignore", divide="ignore"):
+        c, s = _rotation(apq, app, aqq)
+    tau = d / (2.0 * apq)
+    t = np.copysign(1.0, tau) / (np.abs(tau) + np.sqrt(1.0 + tau * tau))
+    ce = 1.0 / np.sqrt(1.0 + t * t)
+    return np.where(wide, ce, c), np.where(wide, t * ce, s)
+
+
+@pytest.mark.parametrize("log_tau", [50, 58, 59, 60, 61, 62, 63, 64, 65, 70, 90, 99, 100, 101, 110])
+def test_rotation_of_a_graded_pair(log_tau):
+    rng = np.random.default_rng(log_tau)
+    apq = rng.normal(size=5000)
+    apq[np.abs(apq) < 1e-3] = 1.0
+    app, aqq = np.zeros(5000), rng.uniform(1.0, 4.0, 5000) * 2.0 ** log_tau
+    c, s = _guarded(apq, app, aqq)
+    assert np.all(s != 0.0)
+    # a_pq is annihilated: t = a_pq / a_qq there, to a few FP32 roundings
+    left = (c * c - s * s) * apq + c * s * (app - aqq)
+    assert np.all(np.abs(left) <= 1e-6 * np.abs(apq))
