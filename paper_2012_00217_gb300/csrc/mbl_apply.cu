@@ -2213,8 +2213,10 @@ __global__ void __launch_bounds__(kThreads) k_pcg_update(uint32_t n, const T *__
 // k = 64: 185 against 190 us; L = 22, k = 32: 301 against 404 us) and stay.
 //
 // A lane's blocks wait for one another, so the launch is cooperative.  Every wait is
-// bounded; on a time-out the lane's fail word is set, its blocks leave, and each writes
-// NaN into w, which the solver reports as MBL_ERR_NUMERIC.
+// bounded; on a time-out, of a barrier or of a staged copy, the lane's fail word is set.  The
+// block that gave up leaves at its next barrier, the others when they wait for it or, at the
+// latest, when they look at the word after the last step, and each writes NaN into w, which
+// the solver reports as MBL_ERR_NUMERIC.
 
 constexpr int kRunThreads = 768;
 constexpr int kRunWarps = kRunThreads / 32;
@@ -2309,6 +2311,7 @@ struct RunShared {
     int cls_p[kLowMaxB + 1], ncls;
     PcgLane lane;
     int ok;
+    int copy_failed;  // a staged copy of this block was given up
     uint32_t tmem;
     __align__(8) uint64_t mbar[kRunSubs];
     unsigned parity[kRunWarps];  // of the waits on mbar, per warp
@@ -2355,16 +2358,16 @@ __device__ __forceinline__ bool lane_barrier(RunShared<T> &sm, unsigned &target)
     if (ASYNC) fence_proxy_async();
     __syncthreads();
     const unsigned nb = sm.lane.nblocks;
-    if (nb == 1) return true;
+    if (nb == 1) return !(ASYNC && sm.copy_failed);
     target += nb;
     if (threadIdx.x == 0) {
         unsigned *bar = sm.lane.counter + 1;
         const unsigned *fail = sm.lane.counter + 3;
         // release: the block's stores of this phase come first; acquire: after the last arrival
         asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(bar) : "memory");
-        int ok = 1;
+        int ok = ASYNC && sm.copy_failed ? 0 : 1;
         const long long t0 = clock64();
-        for (unsigned polls = 1; ld_relaxed(bar) < target; ++polls) {
+        for (unsigned polls = 1; ok && ld_relaxed(bar) < target; ++polls) {
             if (polls % 256u) continue;
             if (ld_relaxed(fail)) ok = 0;
             else if (clock64() - t0 > kLaneWaitCycles) {
@@ -2499,6 +2502,21 @@ __device__ __forceinline__ void run_cache_jobs(RunShared<T> &sm, const RunShare 
     }
 }
 
+// Barrier `id` of a staging group, with the conjunction of what its threads bring.
+__device__ __forceinline__ bool group_all(int id, bool mine)
+{
+    uint32_t all;
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\t"
+        "setp.ne.u32 p, %1, 0;\n\t"
+        "bar.red.and.pred q, %2, %3, p;\n\t"
+        "selp.u32 %0, 1, 0, q;\n\t}"
+        : "=r"(all)
+        : "r"((uint32_t)mine), "r"(id), "r"(kThreads)
+        : "memory");
+    return all != 0;
+}
+
 // The product of this block's jobs: Y = (H - sigma) X and, per column, the warp's sum of
 // y.y (kPcgT) or x.y (kDot), or q = (H - sigma) X, R -= alpha q and the sum of R.(M^-1 R)
 // (kPcgQ), into sm.red.  Staged: a group of 256 threads takes whole tiles, one at a time: the other groups
@@ -2568,9 +2586,11 @@ __device__ __noinline__ void run_product()
         if (wsub == 0 && sh.count > 0) issue(0);
 #pragma unroll 1
         for (uint32_t i = 0; i < sh.count; ++i) {
-            if (!mbar_wait_bounded(mbar, parity)) {
+            const bool got = mbar_wait_bounded(mbar, parity);
+            if (!got) {
                 // wait once more so that no copy is left in flight, and fail the lane
                 mbar_wait_bounded(mbar, parity);
+                sm.copy_failed = 1;
                 atomicExch(Ln.counter + 3, 1u);
             }
             parity ^= 1u;
@@ -2582,15 +2602,17 @@ __device__ __noinline__ void run_product()
             const T *Xt = reinterpret_cast<const T *>(buf);
             const LowRec *rp =
                 RS ? reinterpret_cast<const LowRec *>(buf + je * (uint32_t)(K * sizeof(T))) : tbl + sm.spref[p];
+            const bool whole = __all_sync(0xffffffffu, got);  // else this warp's rows are left out
 #pragma unroll 1
-            for (uint32_t j0 = wsub * RPW; j0 < je; j0 += RPB) {
+            for (uint32_t j0 = wsub * RPW; whole && j0 < je; j0 += RPB) {
                 const uint32_t j = j0 + grp;
                 tile_row_pass<T, V, NB, MODE, RS>(cp, B, X, K, Xt, K, rp, min(j, je - 1u), j < je, job.meta, sm.tab,
                                               hdelta, t0, thi, sup, sdn, col, Y, K, R, dinv, sm.alpha, part,
                                               nullptr, nullptr);
             }
-            // every read of this buffer and job is done before they are filled again
-            asm volatile("bar.sync %0, %1;" ::"r"(1 + sub), "r"(kThreads) : "memory");
+            // every read of this buffer and job is done before they are filled again; a group with
+            // an incomplete tile stops here, all of it
+            if (!group_all(1 + sub, whole)) break;
             if (wsub == 0 && i + 1 < sh.count) issue(i + 1);
         }
         if (lane == 0) sm.parity[warp] = parity;
@@ -2736,6 +2758,7 @@ __device__ __forceinline__ void run_setup(const PcgLane *src)
     load_binom(sm.binom);
     if (STAGED && threadIdx.x < kRunSubs) mbar_init(&sm.mbar[threadIdx.x], 1);
     if (threadIdx.x < kRunWarps) sm.parity[threadIdx.x] = 0;
+    if (threadIdx.x == 0) sm.copy_failed = 0;
     __syncthreads();
     build_field_tables<T>(sm.tab, Ln.cp);
     if (threadIdx.x == 0) {
@@ -2854,6 +2877,12 @@ __global__ void __launch_bounds__(kRunThreads, 1)
         if (w_tmem) run_update<T, K, true>(row_b, row_e, tmem);
         else run_update<T, K, false>(row_b, row_e, 0u);
         if (step + 1 < steps && !(ok = lane_barrier<STAGED>(sm, target))) break;
+    }
+    if (ok) {
+        // whatever a block gave up in came before its last arrival
+        if (threadIdx.x == 0) sm.ok = ld_relaxed(Ln.counter + 3) == 0u;
+        __syncthreads();
+        ok = sm.ok != 0;
     }
     if (w_tmem && ok) run_move_w<T, K, false>(row_b, row_e, tmem);
     if (!ok && row_b < row_e && threadIdx.x < K)
