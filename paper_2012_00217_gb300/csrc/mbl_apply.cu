@@ -3287,16 +3287,38 @@ static int lane_bytes_for(int L, int K, size_t es)
     return size_lane_bytes(K, es);
 }
 
+// Items that the tiled kernels go through for chunks of `chunk` rows: those of all tiles, with
+// and without rows.
+static int64_t tiled_items(int L, int B, uint32_t chunk)
+{
+    return ((int64_t)1 << (L - B)) * (int64_t)((host_binom(B, B / 2) + chunk - 1) / chunk);
+}
+
 // Rows per work item of the tiled kernels: `most`, or as few as still give every resident
 // warp an item when the sector is small, so that its rows are not passed over one after
 // another by a few warps (a pass is a chain of three dependent loads).  Measured on GB300
 // against always `most`: FP32 L = 12, k = 8 8.8 -> 5.3 us, L = 16, k = 16 11.1 -> 6.6 us; FP64
 // L = 14, k = 16 42 -> 16 us, L = 18, k = 32 90 -> 72 us.
-static uint32_t chunk_rows(uint32_t n, uint32_t rows_per_pass, int resident_warps, uint32_t most)
+// An item without rows costs a warp about 0.17 us, and with few up spins on a long chain nearly
+// all are of that kind, so chunks shrink only to where warp_items of all items come on a warp:
+// 16, or nine for four columns in FP64, whose passes take longer.  `most` / shrunk, us, FP32: L = 20,
+// n_up = 17, k = 32 (15 a warp) 9.1 / 7.7; L = 22, n_up = 3, k = 32 (30) 9.4 / 12.3; L = 28,
+// n_up = 3, k = 64 (3880) 102 / 640.  FP64: L = 22, n_up = 18, k = 64 (60) 100 / 60; L = 24,
+// n_up = 2, k = 8 (60) 18 / 25; L = 28, n_up = 3, k = 64 (3880) 181 / 719.
+static uint32_t small_chunk(const ChainParams &cp, uint32_t rows_per_pass, int resident_warps, uint32_t most)
 {
     const uint64_t pass = (uint64_t)rows_per_pass * (uint64_t)resident_warps;
-    const uint64_t rows = rows_per_pass * ((n + pass - 1) / pass);
+    const uint64_t rows = rows_per_pass * ((host_binom(cp.L, cp.n_up) + pass - 1) / pass);
     return rows < most ? (uint32_t)rows : most;
+}
+
+static int64_t warp_items(int k, size_t es) { return es == 8 && k > 8 ? 9 * k / 4 : 16; }
+
+static uint32_t chunk_rows(const ChainParams &cp, int B, int k, size_t es, uint32_t rows_per_pass, int resident_warps,
+                           uint32_t most)
+{
+    const uint32_t rows = small_chunk(cp, rows_per_pass, resident_warps, most);
+    return tiled_items(cp.L, B, rows) <= warp_items(k, es) * resident_warps ? rows : most;
 }
 
 // per_sm: resident blocks per SM of the kernel, with its preferred L1 share set.
@@ -3325,12 +3347,11 @@ static cudaError_t launch_tiled_lb(const ChainParams &cp, int B, const T *X, int
     int64_t grid = (int64_t)num_sms() * tiled_blocks_per_sm<T, K, MODE, LB, true>();
     const uint32_t CH = ordered || MODE != kPlain
                             ? (uint32_t)Lay::CH
-                            : chunk_rows(host_binom(cp.L, cp.n_up), 32 / Lay::G, (int)grid * kWarps, Lay::CH);
+                            : chunk_rows(cp, B, K, sizeof(T), 32 / Lay::G, (int)grid * kWarps, Lay::CH);
     const bool full = CH == (uint32_t)Lay::CH;
     if constexpr (MODE == kPlain)
         if (!full) grid = (int64_t)num_sms() * tiled_blocks_per_sm<T, K, MODE, LB, false>();
-    const int64_t items = ((int64_t)1 << (cp.L - B)) * (int64_t)((host_binom(B, B / 2) + CH - 1) / CH);
-    const int64_t need = (items + kWarps - 1) / kWarps;
+    const int64_t need = (tiled_items(cp.L, B, CH) + kWarps - 1) / kWarps;
     if (ordered || grid > need) grid = need;
     note_launch();
     if constexpr (MODE == kPlain)
@@ -3554,13 +3575,29 @@ static int any_vector(const void *X, int64_t ldx, const void *Y, int64_t ldy, in
     return 1;
 }
 
+// Rows per item of the any-width kernel where a warp takes rpw rows at a time, at most.
+static uint32_t any_chunk(int rpw) { return (uint32_t)(MBL_CH_PASSES * rpw > 32 ? MBL_CH_PASSES * rpw : 32); }
+
 // The any-width kernel does a row's index work in each of its lanes: it pays where a warp
 // takes two rows or more at a time (FP32, L = 20: k = 24 77 -> 29 us; k = 32 with an odd
 // leading dimension, a row a pass, 139 against the row-a-warp kernel's 78 us).
+// And not where its items without rows cost more than that: about 50 ps each over all warps,
+// against 260 ps that the row-a-warp kernel takes longer for a row, so up to 4 items a row; or
+// up to 64 a warp, less than the 17 us of that kernel's smallest launch.  FP64 sectors whose
+// chunks should shrink and may not (chunk_rows) stay with the row-a-warp kernel too.  us,
+// row-a-warp / any width: FP32 k = 20 L = 24, n_up = 5 34 / 29, L = 28, n_up = 5 39 / 128,
+// L = 32, n_up = 2 19 / 6605; FP64 k = 20 L = 24, n_up = 5 62 / 81.
 template <typename T>
-static bool any_width_ok(const void *X, int64_t ldx, const void *Y, int64_t ldy, int k)
+static bool any_width_ok(const ChainParams &cp, int B, const void *X, int64_t ldx, const void *Y, int64_t ldy, int k)
 {
-    return k / any_vector<T>(X, ldx, Y, ldy, k) <= 16;
+    const int G = k / any_vector<T>(X, ldx, Y, ldy, k);
+    if (G > 16) return false;
+    const uint32_t rpw = 32u / (uint32_t)G, most = any_chunk((int)rpw);
+    const int warps = num_sms() * MBL_TILED_MIN_BLOCKS * kWarps;
+    const uint32_t chunk = chunk_rows(cp, B, k, sizeof(T), rpw, warps, most);
+    if (sizeof(T) == 8 && chunk != small_chunk(cp, rpw, warps, most)) return false;
+    const int64_t items = tiled_items(cp.L, B, chunk);
+    return items <= (int64_t)64 * warps || items <= 4 * (int64_t)host_binom(cp.L, cp.n_up);
 }
 
 template <typename T, int V>
@@ -3576,11 +3613,8 @@ static cudaError_t launch_any_v(const ChainParams &cp, int B, const T *X, int64_
     }();
     const int RPW = 32 / (k / V);
     const int64_t cap = (int64_t)num_sms() * per_sm;
-    const uint32_t rmax = host_binom(B, B / 2);
-    const uint32_t CH = chunk_rows(host_binom(cp.L, cp.n_up), (uint32_t)RPW, (int)cap * kWarps,
-                                   (uint32_t)(MBL_CH_PASSES * RPW > 32 ? MBL_CH_PASSES * RPW : 32));
-    const int64_t items = ((int64_t)1 << (cp.L - B)) * (int64_t)((rmax + CH - 1) / CH);
-    const int64_t need = (items + kWarps - 1) / kWarps;
+    const uint32_t CH = chunk_rows(cp, B, k, sizeof(T), (uint32_t)RPW, (int)cap * kWarps, any_chunk(RPW));
+    const int64_t need = (tiled_items(cp.L, B, CH) + kWarps - 1) / kWarps;
     note_launch();
     kern<<<(int)(need < cap ? need : cap), kThreads, 0, st>>>(cp, B, CH, X, ldx, Y, ldy, k);
     return cudaGetLastError();
@@ -3636,7 +3670,7 @@ static int dispatch_plain(const ChainParams &cp, const T *X, int64_t ldx, T *Y, 
     } else {
         done = false;
     }
-    if (!done && B >= 2 && any_width_ok<T>(X, ldx, Y, ldy, k) && lowtab_usable(B, st)) {
+    if (!done && B >= 2 && any_width_ok<T>(cp, B, X, ldx, Y, ldy, k) && lowtab_usable(B, st)) {
         e = launch_any<T>(cp, B, X, ldx, Y, ldy, k, st);
     } else if (!done) {
         const size_t sm = apply_smem_bytes<T>();
