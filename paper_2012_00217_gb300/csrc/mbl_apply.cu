@@ -1979,9 +1979,9 @@ static bool lowtab_usable(int B, cudaStream_t st)
     return cudaStreamIsCapturing(st, &status) == cudaSuccess && status == cudaStreamCaptureStatusNone;
 }
 
-// Untiled product (chains of fewer than four sites, tile bits -1, or a capture that meets a
-// tile width for the first time) of any block width and alignment: one warp per row, lanes
-// stride the columns.  Plain product only.
+// Product of any block width and alignment, a row a warp, lanes striding the columns: untiled
+// chains (fewer than four sites, tile bits -1), a capture that meets a tile width for the first
+// time, and where any_width_ok finds it the faster one.  Plain product only.
 template <typename T>
 __global__ void __launch_bounds__(kThreads) k_apply_generic(ChainParams cp, const T *__restrict__ X,
                                                             int64_t ldx, T *__restrict__ Y, int64_t ldy,
@@ -3578,26 +3578,62 @@ static int any_vector(const void *X, int64_t ldx, const void *Y, int64_t ldy, in
 // Rows per item of the any-width kernel where a warp takes rpw rows at a time, at most.
 static uint32_t any_chunk(int rpw) { return (uint32_t)(MBL_CH_PASSES * rpw > 32 ? MBL_CH_PASSES * rpw : 32); }
 
-// The any-width kernel does a row's index work in each of its lanes: it pays where a warp
-// takes two rows or more at a time (FP32, L = 20: k = 24 77 -> 29 us; k = 32 with an odd
-// leading dimension, a row a pass, 139 against the row-a-warp kernel's 78 us).
-// And not where its items without rows cost more than that: about 50 ps each over all warps,
-// against 260 ps that the row-a-warp kernel takes longer for a row, so up to 4 items a row; or
-// up to 64 a warp, less than the 17 us of that kernel's smallest launch.  FP64 sectors whose
-// chunks should shrink and may not (chunk_rows) stay with the row-a-warp kernel too.  us,
-// row-a-warp / any width: FP32 k = 20 L = 24, n_up = 5 34 / 29, L = 28, n_up = 5 39 / 128,
-// L = 32, n_up = 2 19 / 6605; FP64 k = 20 L = 24, n_up = 5 62 / 81.
+// Share of the tiled rows, 2^(L-B) tiles of C(B, B/2), that the sector has: 0.74 to 0.84 for a
+// half-filled chain of 20 to 26 sites, 0.57 two up spins away from that.
+static double tile_fill(const ChainParams &cp, int B)
+{
+    return (double)host_binom(cp.L, cp.n_up) / ((double)((int64_t)1 << (cp.L - B)) * (double)host_binom(B, B / 2));
+}
+
+static bool compiled_width(int k) { return k == 1 || k == 2 || k == 4 || k == 8 || k == 16 || k == 32 || k == 64; }
+
+// Whether the any-width kernel takes a product, against k_apply (compiled widths whose rows are
+// aligned to 16 bytes, not to the tiled kernels' lanes) and the row-a-warp kernel.
+//
+// It does a row's index work in each of its lanes: a warp has to take two rows or more at a
+// time (FP32, L = 20, k = 32 with an odd leading dimension, a row a pass: 139 against 78 us).
+//
+// Its items without rows cost about 50 ps each over all warps, against 260 ps that the
+// row-a-warp kernel takes longer for a row: up to 4 items a row, or up to 64 a warp, less than
+// the 17 us of that kernel's smallest launch.  FP64 sectors whose chunks should shrink and may
+// not (chunk_rows) are left out too.  us, row-a-warp / any width: FP32 k = 20 L = 24, n_up = 5
+// 34 / 29, L = 28, n_up = 5 39 / 128, L = 32, n_up = 2 19 / 6605; FP64 k = 20 L = 24, n_up = 5
+// 62 / 81.
+//
+// Up to six rows a warp it always pays (0.1 to 0.9 of the others' time).  Beyond that, in FP32,
+// for all but
+//   - k_apply's widths in sectors off the middle (k = 16, ld = 20: L = 20, n_up = 10 24 / 30 us,
+//     n_up = 8 24 / 21);
+//   - narrow vectors with two rows a pass, off the middle (k = 16, ld = 17: L = 20, n_up = 8 63 /
+//     45 us).
+// In FP64 the pipe decides: V additions for rpw rows against ceil(k / 32) for one, q the ratio,
+// about 1.6 q of the row-a-warp kernel's time when full, and more as the tiles get emptier (us,
+// any width / row-a-warp, L = 20: n_up = 10 k = 12 111 / 199, k = 24 225 / 199, k = 22 336 / 198;
+// n_up = 8 k = 20 180 / 131).
 template <typename T>
 static bool any_width_ok(const ChainParams &cp, int B, const void *X, int64_t ldx, const void *Y, int64_t ldy, int k)
 {
-    const int G = k / any_vector<T>(X, ldx, Y, ldy, k);
+    const int V = any_vector<T>(X, ldx, Y, ldy, k), G = k / V;
     if (G > 16) return false;
     const uint32_t rpw = 32u / (uint32_t)G, most = any_chunk((int)rpw);
     const int warps = num_sms() * MBL_TILED_MIN_BLOCKS * kWarps;
     const uint32_t chunk = chunk_rows(cp, B, k, sizeof(T), rpw, warps, most);
     if (sizeof(T) == 8 && chunk != small_chunk(cp, rpw, warps, most)) return false;
+    const double n = (double)host_binom(cp.L, cp.n_up), fill = tile_fill(cp, B);
     const int64_t items = tiled_items(cp.L, B, chunk);
-    return items <= (int64_t)64 * warps || items <= 4 * (int64_t)host_binom(cp.L, cp.n_up);
+    if (items > (int64_t)64 * warps && (double)items > 4.0 * n) return false;
+    if (n <= 6.0 * warps) return true;
+    const bool other = compiled_width(k) && vec_ok<T>(X, ldx, k) && vec_ok<T>(Y, ldy, k);
+    if (sizeof(T) == 4) {
+        if (other) return fill >= 0.7 || (fill >= 0.4 && (n <= 15.0 * warps || n >= 64.0 * warps));
+        if (rpw > 2 || V >= 4) return true;
+        return fill >= 0.7 || (fill >= 0.4 && (V == 2 || n <= 24.0 * warps));
+    }
+    const double q = (double)V / (double)(rpw * (uint32_t)((k + 31) / 32));
+    if (q <= 0.25) return true;
+    if (other && k == 16) return fill >= 0.7;
+    if (q <= 0.4) return fill >= 0.4 || (fill >= 0.1 && n >= 40.0 * warps);
+    return fill >= 0.4 && q < 1.0 && n <= 15.0 * warps;
 }
 
 template <typename T, int V>
@@ -3642,10 +3678,10 @@ static int dispatch_plain(const ChainParams &cp, const T *X, int64_t ldx, T *Y, 
     Reduce rd{};
     const int grid = apply_grid(n, 8);
     cudaError_t e = cudaSuccess;
-    bool done = true;
     const int B = tile_bits_for(cp.L, k, sizeof(T));
     const int lb = lane_bytes_for(cp.L, k, sizeof(T));
-    if (B >= 2 && vec_ok_wide<T>(X, ldx, k, lb) && vec_ok_wide<T>(Y, ldy, k, lb)) {
+    const bool compiled = compiled_width(k);
+    if (B >= 2 && compiled && vec_ok_wide<T>(X, ldx, k, lb) && vec_ok_wide<T>(Y, ldy, k, lb)) {
         switch (k) {
         case 1: e = launch_tiled<T, 1, kPlain>(cp, B, X, ldx, Y, ldy, nullptr, nullptr, ps, rd, st); break;
         case 2: e = launch_tiled<T, 2, kPlain>(cp, B, X, ldx, Y, ldy, nullptr, nullptr, ps, rd, st); break;
@@ -3653,10 +3689,13 @@ static int dispatch_plain(const ChainParams &cp, const T *X, int64_t ldx, T *Y, 
         case 8: e = launch_tiled<T, 8, kPlain>(cp, B, X, ldx, Y, ldy, nullptr, nullptr, ps, rd, st); break;
         case 16: e = launch_tiled<T, 16, kPlain>(cp, B, X, ldx, Y, ldy, nullptr, nullptr, ps, rd, st); break;
         case 32: e = launch_tiled<T, 32, kPlain>(cp, B, X, ldx, Y, ldy, nullptr, nullptr, ps, rd, st); break;
-        case 64: e = launch_tiled<T, 64, kPlain>(cp, B, X, ldx, Y, ldy, nullptr, nullptr, ps, rd, st); break;
-        default: done = false;
+        default: e = launch_tiled<T, 64, kPlain>(cp, B, X, ldx, Y, ldy, nullptr, nullptr, ps, rd, st); break;
         }
-    } else if (B < 2 && vec_ok<T>(X, ldx, k) && vec_ok<T>(Y, ldy, k)) {
+    } else if (B >= 2 && any_width_ok<T>(cp, B, X, ldx, Y, ldy, k) && lowtab_usable(B, st)) {
+        e = launch_any<T>(cp, B, X, ldx, Y, ldy, k, st);
+    } else if (compiled && vec_ok<T>(X, ldx, k) && vec_ok<T>(Y, ldy, k) && (B < 2 || sizeof(T) == 4 || k <= 16)) {
+        // wide FP64 rows of a tiled chain are faster a row a warp (L = 20, n_up = 8: k = 32, ld =
+        // 34 289 us here, 132 there)
         switch (k) {
         case 1: e = launch_apply_k<T, 1, kPlain>(cp, X, ldx, Y, ldy, n, nullptr, nullptr, ps, rd, grid, st); break;
         case 2: e = launch_apply_k<T, 2, kPlain>(cp, X, ldx, Y, ldy, n, nullptr, nullptr, ps, rd, grid, st); break;
@@ -3664,15 +3703,9 @@ static int dispatch_plain(const ChainParams &cp, const T *X, int64_t ldx, T *Y, 
         case 8: e = launch_apply_k<T, 8, kPlain>(cp, X, ldx, Y, ldy, n, nullptr, nullptr, ps, rd, grid, st); break;
         case 16: e = launch_apply_k<T, 16, kPlain>(cp, X, ldx, Y, ldy, n, nullptr, nullptr, ps, rd, grid, st); break;
         case 32: e = launch_apply_k<T, 32, kPlain>(cp, X, ldx, Y, ldy, n, nullptr, nullptr, ps, rd, grid, st); break;
-        case 64: e = launch_apply_k<T, 64, kPlain>(cp, X, ldx, Y, ldy, n, nullptr, nullptr, ps, rd, grid, st); break;
-        default: done = false;
+        default: e = launch_apply_k<T, 64, kPlain>(cp, X, ldx, Y, ldy, n, nullptr, nullptr, ps, rd, grid, st); break;
         }
     } else {
-        done = false;
-    }
-    if (!done && B >= 2 && any_width_ok<T>(cp, B, X, ldx, Y, ldy, k) && lowtab_usable(B, st)) {
-        e = launch_any<T>(cp, B, X, ldx, Y, ldy, k, st);
-    } else if (!done) {
         const size_t sm = apply_smem_bytes<T>();
         static const bool attr_set_once = [&]() {
             cudaFuncSetAttribute(k_apply_generic<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);

@@ -1,0 +1,56 @@
+"""Products of widths or alignments without a tiled kernel take the faster of the any-width kernel, the
+compiled untiled kernels and the row-a-warp kernel: the values against the oracle on both sides of
+that choice, and the time against the untiled kernels (tile bits -1: the latter two)."""
+import numpy as np
+import pytest
+
+import workloads as wl
+from oracle import hamiltonian as ham
+
+from test_gpu_parity import _bound
+from test_gpu_sparse_sectors import _time
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+DEV = "cuda:0"
+
+
+@pytest.fixture(scope="module")
+def mbl():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_2012_00217_gb300 as m
+    m.binding.lib()
+    return m
+
+
+# k < 32 and odd leading dimensions: vectors of 1, 2 and 4 elements, two rows a pass and more, FP64
+# pipe ratios from 0.1 to 1, on sectors in and off the middle, from six rows a warp on.  1.25: the
+# spread of the rule's own measurements; the cases it is there for were 1.3 to 2.5
+@pytest.mark.parametrize("L,n_up,k,ld,dtype", [
+    (18, 9, 22, 22, "f64"), (18, 7, 30, 30, "f64"), (19, 8, 28, 28, "f64"), (19, 8, 20, 20, "f64"), (20, 8, 12, 12, "f64"),
+    (20, 10, 24, 24, "f64"), (20, 8, 44, 44, "f64"), (20, 12, 36, 36, "f64"), (20, 8, 16, 17, "f64"), (20, 8, 7, 7, "f64"),
+    (20, 8, 10, 10, "f64"), (20, 8, 32, 34, "f64"), (20, 14, 64, 66, "f64"), (20, 14, 16, 18, "f64"), (20, 10, 16, 18, "f64"),
+    (20, 8, 16, 17, "f32"), (20, 10, 16, 17, "f32"), (20, 14, 22, 22, "f32"), (20, 8, 24, 24, "f32"), (19, 8, 16, 20, "f32"),
+    (20, 14, 32, 36, "f32"), (20, 10, 64, 68, "f32")])
+def test_route(mbl, L, n_up, k, ld, dtype):
+    npt, tdt = (np.float32, torch.float32) if dtype == "f32" else (np.float64, torch.float64)
+    h = wl.fields(L, 6.0, L + k)
+    chain = ham.Chain(L, h, delta=0.8, periodic=True, n_up=n_up)
+    n = ham.sector_dim(L, n_up)
+    Xb = wl.block(n, ld, 3 + k, npt)
+    ref = ham.apply(chain, 0.4, Xb[:, :k].astype(np.float64))
+    X = torch.from_numpy(Xb).to(DEV)[:, :k]
+    Yf = torch.full((n, ld), 77.0, dtype=tdt, device=DEV)
+    Y = Yf[:, :k]
+    mc = mbl.make_chain(L, h, 0.8, True, n_up)
+    mbl.hamiltonian_apply(mc, 0.4, X, Y)
+    assert np.all(np.abs(Y.cpu().numpy().astype(np.float64) - ref) <= _bound(chain, 0.4, Xb[:, :k], npt))
+    assert torch.all(Yf[:, k:] == 77.0)
+    us = _time(mbl, mc, X, Y)
+    mbl.binding.set_product_tile_bits(k, tdt, -1)
+    try:
+        untiled = _time(mbl, mc, X, Y)
+    finally:
+        mbl.binding.set_product_tile_bits(k, tdt, 0)
+    assert us <= 1.25 * untiled, (us, untiled)
