@@ -122,9 +122,10 @@ int mbl_set_product_lane_bytes(int k, int dtype, int bytes);
 /* Tuning: work order of the tiled product for block width k and type dtype.
  * 0 = by size (default, unless mbl_autotune_product chose for this L; of the block's bytes
  * C(L, n_up) * k * element size: FP32 rows of 64 to 256 bytes staged from 16 MiB (256 bytes:
- * 32 MiB), rows of 256 bytes and more ordered from 1 GiB, FP64 rows of 128 bytes and more
- * ordered from 32 MiB, of 128 bytes staged from 16 MiB to there, else persistent; the PCG of
- * a solve has rules of its own), 1 = persistent (a few blocks per SM striding over the tiles), 2 = ordered
+ * 32 MiB; 64 and 256 bytes near half filling only), rows of 256 bytes and more ordered from
+ * 1 GiB, FP64 rows of 128 bytes and more ordered from 32 MiB, of 128 bytes staged from 16 MiB
+ * to there, else persistent; the PCG of a solve has rules of its own), 1 = persistent (a few
+ * blocks per SM striding over the tiles), 2 = ordered
  * (plain products only: one chunk of rows per warp; the hardware dispatches blocks in
  * index order, so the tiles being read advance as a narrow window that stays in L2),
  * 3 = staged (each block copies whole tiles of at most 48 KB into shared memory with bulk

@@ -3216,6 +3216,13 @@ static ProductTune g_tuned[2][8][kMaxL + 1] = {};
 static std::mutex g_tune_mutex;
 static thread_local int t_force_schedule = 0, t_force_lane = 0;
 
+// Share of the tiled rows, 2^(L-B) tiles of C(B, B/2), that a sector has: 0.74 to 0.84 for a
+// half-filled chain of 20 to 26 sites, 0.57 two up spins away from that.
+static double tile_fill(int L, int n_up, int B)
+{
+    return (double)host_binom(L, n_up) / ((double)((int64_t)1 << (L - B)) * (double)host_binom(B, B / 2));
+}
+
 // Work order of a plain tiled product.  Persistent: a grid of a few blocks per SM, each
 // warp striding over the (tile, chunk) items.  Ordered: one item per warp and as many
 // blocks as needed, so the hardware hands out blocks in index order and the tiles in
@@ -3232,6 +3239,10 @@ static thread_local int t_force_schedule = 0, t_force_lane = 0;
 // so FP32 rows of 64 to 256 bytes are staged from 16 MB (256 bytes: 32 MB) and ordered from
 // 1 GiB (256 bytes and wider); FP64 rows of 128 bytes and more are ordered from 32 MB, those
 // of exactly 128 bytes staged from 16 MB to there.
+// Staged blocks take whole tiles as their numbers come, so they lose where the tiles differ much
+// in size: rows of 64 and 256 bytes are staged where the sector fills 0.6 of its tiles (persistent
+// / staged, FP32: k = 16 L = 24, n_up = 11 (0.71) 180 / 188, n_up = 10 (0.56) 145 / 173; k = 64
+// L = 24, n_up = 10 (0.56) 640 / 632, n_up = 7 (0.10) 131 / 233).
 static int size_schedule(int L, int n_up, int K, size_t es)
 {
     const double mb = (double)host_binom(L, n_up) * K * (double)es / (1 << 20);
@@ -3241,7 +3252,10 @@ static int size_schedule(int L, int n_up, int K, size_t es)
         return row == 128 && mb >= 16.0 ? 3 : 1;
     }
     if (row >= 256 && mb >= 1024.0) return 2;
-    return row >= 64 && row <= 256 && mb >= (row == 256 ? 32.0 : 16.0) ? 3 : 1;
+    if (row == 128) return mb >= 16.0 ? 3 : 1;
+    const int B = heuristic_tile_bits(L, K, es);
+    if ((row != 64 && row != 256) || B < 2 || tile_fill(L, n_up, B) < 0.6) return 1;
+    return mb >= (row == 256 ? 32.0 : 16.0) ? 3 : 1;
 }
 
 static int explicit_schedule(int K, size_t es) { return g_schedule[es == 8 ? 1 : 0][kslot(K)]; }
@@ -3578,13 +3592,6 @@ static int any_vector(const void *X, int64_t ldx, const void *Y, int64_t ldy, in
 // Rows per item of the any-width kernel where a warp takes rpw rows at a time, at most.
 static uint32_t any_chunk(int rpw) { return (uint32_t)(MBL_CH_PASSES * rpw > 32 ? MBL_CH_PASSES * rpw : 32); }
 
-// Share of the tiled rows, 2^(L-B) tiles of C(B, B/2), that the sector has: 0.74 to 0.84 for a
-// half-filled chain of 20 to 26 sites, 0.57 two up spins away from that.
-static double tile_fill(const ChainParams &cp, int B)
-{
-    return (double)host_binom(cp.L, cp.n_up) / ((double)((int64_t)1 << (cp.L - B)) * (double)host_binom(B, B / 2));
-}
-
 static bool compiled_width(int k) { return k == 1 || k == 2 || k == 4 || k == 8 || k == 16 || k == 32 || k == 64; }
 
 // Whether the any-width kernel takes a product, against k_apply (compiled widths whose rows are
@@ -3619,7 +3626,7 @@ static bool any_width_ok(const ChainParams &cp, int B, const void *X, int64_t ld
     const int warps = num_sms() * MBL_TILED_MIN_BLOCKS * kWarps;
     const uint32_t chunk = chunk_rows(cp, B, k, sizeof(T), rpw, warps, most);
     if (sizeof(T) == 8 && chunk != small_chunk(cp, rpw, warps, most)) return false;
-    const double n = (double)host_binom(cp.L, cp.n_up), fill = tile_fill(cp, B);
+    const double n = (double)host_binom(cp.L, cp.n_up), fill = tile_fill(cp.L, cp.n_up, B);
     const int64_t items = tiled_items(cp.L, B, chunk);
     if (items > (int64_t)64 * warps && (double)items > 4.0 * n) return false;
     if (n <= 6.0 * warps) return true;

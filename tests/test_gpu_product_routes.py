@@ -54,3 +54,21 @@ def test_route(mbl, L, n_up, k, ld, dtype):
     finally:
         mbl.binding.set_product_tile_bits(k, tdt, 0)
     assert us <= 1.25 * untiled, (us, untiled)
+
+
+@pytest.mark.parametrize("L,n_up,k", [(24, 10, 16), (24, 7, 64), (22, 8, 16), (22, 15, 64), (22, 11, 16), (22, 11, 64)])
+def test_work_order_off_the_middle(mbl, L, n_up, k):
+    """The default order against the two it chooses from: whole tiles a block lose up to twice the
+    time where the tiles' sizes differ."""
+    n = ham.sector_dim(L, n_up)
+    X = torch.randn(n, k, dtype=torch.float32, device=DEV)
+    Y = torch.empty_like(X)
+    mc = mbl.make_chain(L, wl.fields(L, 6.0, L + k), 1.0, False, n_up)
+    us = []
+    try:
+        for order in (0, 1, 3):
+            mbl.binding.set_product_schedule(k, torch.float32, order)
+            us.append(_time(mbl, mc, X, Y))
+    finally:
+        mbl.binding.set_product_schedule(k, torch.float32, 0)
+    assert us[0] <= 1.12 * min(us[1:]), us
