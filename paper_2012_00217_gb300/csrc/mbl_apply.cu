@@ -3359,9 +3359,13 @@ static cudaError_t launch_tiled_lb(const ChainParams &cp, int B, const T *X, int
     // epilogues keep one partial per block in a buffer sized for the persistent grid
     const bool ordered = MODE == kPlain && schedule_for(cp.L, cp.n_up, K, sizeof(T)) == 2;
     int64_t grid = (int64_t)num_sms() * tiled_blocks_per_sm<T, K, MODE, LB, true>();
-    const uint32_t CH = ordered || MODE != kPlain
-                            ? (uint32_t)Lay::CH
-                            : chunk_rows(cp, B, K, sizeof(T), 32 / Lay::G, (int)grid * kWarps, Lay::CH);
+    uint32_t CH = ordered || MODE != kPlain
+                      ? (uint32_t)Lay::CH
+                      : chunk_rows(cp, B, K, sizeof(T), 32 / Lay::G, (int)grid * kWarps, Lay::CH);
+    // FP32 chunks more than half as large as Lay::CH, and so of a size known at run time only, lose
+    // (three quarters of it, FP32: L = 19, n_up = 8, k = 32 16.7 -> 18.6 us, L = 20, n_up = 9, k = 16
+    // 17.9 -> 20.6 us; in FP64 they gain 7 %)
+    if (sizeof(T) == 4 && 2 * CH > (uint32_t)Lay::CH) CH = Lay::CH;
     const bool full = CH == (uint32_t)Lay::CH;
     if constexpr (MODE == kPlain)
         if (!full) grid = (int64_t)num_sms() * tiled_blocks_per_sm<T, K, MODE, LB, false>();

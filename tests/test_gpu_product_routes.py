@@ -72,3 +72,21 @@ def test_work_order_off_the_middle(mbl, L, n_up, k):
     finally:
         mbl.binding.set_product_schedule(k, torch.float32, 0)
     assert us[0] <= 1.12 * min(us[1:]), us
+
+
+@pytest.mark.parametrize("L,n_up,k", [(19, 8, 32), (20, 9, 16), (19, 8, 64), (22, 6, 32), (18, 9, 32), (20, 8, 16)])
+def test_chunks_near_the_largest(mbl, L, n_up, k):
+    """Sectors a little too small for chunks of the largest size, against the ordered order, which
+    always takes those."""
+    n = ham.sector_dim(L, n_up)
+    X = torch.randn(n, k, dtype=torch.float32, device=DEV)
+    Y = torch.empty_like(X)
+    mc = mbl.make_chain(L, wl.fields(L, 6.0, L + k), 1.0, False, n_up)
+    us = []
+    try:
+        for order in (1, 2):
+            mbl.binding.set_product_schedule(k, torch.float32, order)
+            us.append(_time(mbl, mc, X, Y))
+    finally:
+        mbl.binding.set_product_schedule(k, torch.float32, 0)
+    assert us[0] <= 1.05 * us[1], us
