@@ -3270,14 +3270,19 @@ static int schedule_for(int L, int n_up, int K, size_t es)
     return size_schedule(L, n_up, K, es);
 }
 
-// Work order of the PCG launches (the vectors exceed L2 there): staged for rows of 128 bytes
-// and more.  us a step, persistent / staged: FP32 L = 22, k = 32 343 / 297, k = 64 683 / 563,
-// L = 24, k = 64 2903 / 2365; FP64 L = 20, k = 32 596 / 567.
+// Work order of the PCG launches (the vectors exceed L2 there): staged for rows of 128 bytes and
+// more where the sector fills 0.4 of its tiles, in FP64 up to blocks of 100 MB.  us a step,
+// persistent / staged: FP32 L = 22, k = 32 343 / 297, k = 64 683 / 563, L = 24, k = 64 2903 / 2365,
+// n_up = 10 (0.56) 2038 / 1863, n_up = 9 (0.37) 1417 / 1487, n_up = 7 (0.10) 443 / 655; FP64 L = 20,
+// k = 32 594 / 566, L = 22, n_up = 10 (158 MB) 1956 / 2009, n_up = 7 (0.19) 736 / 1032.
 static int pcg_schedule(int L, int n_up, int K, size_t es)
 {
     const int o = explicit_schedule(K, es);
     if (o) return o;
-    return K * (int)es >= 128 && (double)host_binom(L, n_up) * K * (double)es >= 16.0 * (1 << 20) ? 3 : 1;
+    const double mb = (double)host_binom(L, n_up) * K * (double)es / (1 << 20);
+    const int B = heuristic_tile_bits(L, K, es);
+    if (K * (int)es < 128 || mb < 16.0 || B < 2 || tile_fill(L, n_up, B) < 0.4) return 1;
+    return es == 8 && mb > 100.0 ? 1 : 3;
 }
 
 template <int MODE>
