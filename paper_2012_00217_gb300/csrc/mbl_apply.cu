@@ -3801,13 +3801,14 @@ static uint32_t run_rows_per_pass(int K, size_t es)
 }
 
 // Whether a lane's products take whole tiles through shared memory: rows of 128 bytes from
-// 16 MB, unless the switch or the autotuner says otherwise (L = 18, k = 64: 48.9 us a step in
-// chunks, 50.0 staged; FP64 301 and 316; L = 20, k = 32: 87 and 82).
+// 16 MB, unless the switch says otherwise (the autotuner's choice is the plain product's;
+// L = 18, k = 64: 48.9 us a step in chunks, 50.0 staged; FP64 301 and 316; L = 20, k = 32: 87 and
+// 82).
 static bool run_staged(int L, int n_up, int K, size_t es)
 {
-    const int o = explicit_schedule(K, es), a = g_tuned[es == 8 ? 1 : 0][kslot(K)][L].schedule;
+    const int o = explicit_schedule(K, es);
     if ((K * (int)es) % 16 != 0) return false;
-    if (o || a) return (o ? o : a) == 3;
+    if (o) return o == 3;
     return K * (int)es == 128 && (double)host_binom(L, n_up) * K * (double)es >= 16.0 * (1 << 20);
 }
 
