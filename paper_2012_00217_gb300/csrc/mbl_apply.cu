@@ -3800,16 +3800,21 @@ static uint32_t run_rows_per_pass(int K, size_t es)
     return 32u / (uint32_t)(row >= lb ? row / lb : 1);
 }
 
-// Whether a lane's products take whole tiles through shared memory: rows of 128 bytes from
-// 16 MB, unless the switch says otherwise (the autotuner's choice is the plain product's;
-// L = 18, k = 64: 48.9 us a step in chunks, 50.0 staged; FP64 301 and 316; L = 20, k = 32: 87 and
-// 82).
+// Whether a lane's products take whole tiles through shared memory: FP32 rows of 64 to 256 bytes
+// from 20 MB where the sector fills 0.8 of its tiles (of tiles of equal size more are in flight),
+// unless the switch says otherwise; the autotuner's choice is the plain product's.  us a step,
+// chunks / staged: FP32 L = 20, k = 32 83.9 / 79.0, n_up = 9 (fill 0.76) 75.7 / 77.0; L = 19, k = 64
+// 83.2 / 77.2; L = 21, k = 16 85.9 / 82.7, n_up = 9 (0.67) 70.6 / 71.8; L = 24, n_up = 6, k = 32
+// (0.04) 61 / 123; below 12 MB 1 to 6 % slower; k = 8 L = 22 86.4 / 91.1.  FP64 L = 20, k = 16
+// 284 / 294, L = 18, k = 64 296 / 312, L = 19, k = 32 293 / 281.
 static bool run_staged(int L, int n_up, int K, size_t es)
 {
-    const int o = explicit_schedule(K, es);
-    if ((K * (int)es) % 16 != 0) return false;
+    const int o = explicit_schedule(K, es), row = K * (int)es;
+    if (row % 16 != 0) return false;
     if (o) return o == 3;
-    return K * (int)es == 128 && (double)host_binom(L, n_up) * K * (double)es >= 16.0 * (1 << 20);
+    const int B = heuristic_tile_bits(L, K, es);
+    return es == 4 && row >= 64 && row <= 256 && B >= 2 && tile_fill(L, n_up, B) >= 0.8 &&
+           (double)host_binom(L, n_up) * K * (double)es >= 20.0 * (1 << 20);
 }
 
 static int run_staged_bits(int L, int K, size_t es)

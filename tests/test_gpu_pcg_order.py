@@ -1,4 +1,4 @@
-"""The PCG steps of a solve whose vectors exceed L2, in sectors on and off the middle: the default work
+"""The PCG steps of a solve, resident and beyond L2, in sectors on and off the middle: the default work
 order against the two it chooses from."""
 import pytest
 
@@ -11,7 +11,9 @@ DEV = "cuda:0"
 
 
 @pytest.mark.parametrize("L,n_up,k,mode", [(24, 7, 64, 1), (23, 8, 32, 1), (22, 9, 64, 1), (22, 11, 32, 1), (22, 7, 32, 0),
-                                           (22, 10, 32, 0), (20, 10, 32, 0), (23, 8, 16, 0)])
+                                           (22, 10, 32, 0), (20, 10, 32, 0), (23, 8, 16, 0),
+                                           (20, 10, 32, 1), (20, 9, 32, 1), (19, 9, 64, 1), (21, 10, 16, 1), (24, 6, 32, 1),
+                                           (22, 7, 32, 1), (20, 9, 16, 0), (18, 9, 64, 0)])
 def test_pcg_order(L, n_up, k, mode):
     if not torch.cuda.is_available():
         pytest.skip("no CUDA device")
