@@ -303,7 +303,8 @@ int mbl_lobpcg_solve_noalloc(const mbl_chain *chain, double sigma, const mbl_lob
  * a time, and all lanes advance in lock step on `stream`, one LOBPCG iteration per round:
  * the steps before and after the preconditioner are enqueued lane by lane, and the
  * pcg_iters PCG steps of all advancing lanes run in cooperative launches of up to 64 steps,
- * every lane on its own share of the SMs.  When a lane's problem converges (or reaches max_iter) its results are
+ * every lane on its own share of the SMs (where such a launch does not fit, in a context
+ * that has a part of the device's SMs, every lane runs its own launches of single steps).  When a lane's problem converges (or reaches max_iter) its results are
  * written and it takes the next problem.  The host synchronises `stream` once per round
  * to read the lanes' status words.  With opts->use_graph, each lane's steps before and
  * after the preconditioner are captured once per problem as two small CUDA graphs and

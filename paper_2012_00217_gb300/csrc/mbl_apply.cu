@@ -3944,46 +3944,27 @@ int lanczos_run(const ChainParams &cp, uint32_t n, double *u, double *next, doub
     if (max_blocks > (uint32_t)kRunMaxBlocks) max_blocks = kRunMaxBlocks;
     run_split(o, 1, 8, max_blocks < 1 ? 1 : max_blocks);
     o.items = (uint32_t)run_items(cp.L, cp.n_up, o.B, o.chunk);
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3(o.nblocks);
-    cfg.blockDim = dim3(kRunThreads);
-    cfg.dynamicSmemBytes = run_stage_offset<double>();
-    cfg.stream = st;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeCooperative;
-    at[0].val.cooperative = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    note_launch();
-    return cudaLaunchKernelEx(&cfg, k_lz_run, o, j0, steps) == cudaSuccess ? MBL_OK : MBL_ERR_CUDA;
+    void *args[] = {&o, &j0, &steps};
+    return cooperative_launch((const void *)k_lz_run, o.nblocks, kRunThreads, run_stage_offset<double>(), args, st);
 }
 
 template <typename T, int K, bool STAGED>
-static cudaError_t pcg_run_launch(const PcgLane *one, const PcgLane *lanes_dev, int nlanes, uint32_t blocks,
-                                  size_t dyn, int steps, cudaStream_t st)
+static int pcg_run_launch(const PcgLane *one, const PcgLane *lanes_dev, int nlanes, uint32_t blocks, size_t dyn,
+                          int steps, cudaStream_t st)
 {
     auto kern = k_pcg_run<T, K, STAGED>;
     constexpr size_t state = run_stage_offset<T>();
     static const cudaError_t attr = cudaFuncSetAttribute(
         kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(state + (STAGED ? kRunSubs * (kRunStageBytes + kRunStageBytes / 4) : 0)));
-    if (attr != cudaSuccess) return attr;
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3(blocks);
-    cfg.blockDim = dim3(kRunThreads);
-    cfg.dynamicSmemBytes = state + dyn;
-    cfg.stream = st;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeCooperative;
-    at[0].val.cooperative = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    note_launch();
-    return cudaLaunchKernelEx(&cfg, kern, one ? *one : PcgLane{}, lanes_dev, nlanes, steps);
+    if (attr != cudaSuccess) return MBL_ERR_CUDA;
+    PcgLane lane = one ? *one : PcgLane{};
+    void *args[] = {&lane, &lanes_dev, &nlanes, &steps};
+    return cooperative_launch((const void *)kern, blocks, kRunThreads, state + dyn, args, st);
 }
 
 template <typename T, int K>
-static cudaError_t pcg_run_k(const PcgLane *one, const PcgLane *lanes_dev, int nlanes, uint32_t blocks,
-                             uint32_t stage_bytes, int steps, cudaStream_t st)
+static int pcg_run_k(const PcgLane *one, const PcgLane *lanes_dev, int nlanes, uint32_t blocks, uint32_t stage_bytes,
+                     int steps, cudaStream_t st)
 {
     if (stage_bytes)
         return pcg_run_launch<T, K, true>(one, lanes_dev, nlanes, blocks, (size_t)stage_bytes * kRunSubs, steps, st);
@@ -3998,7 +3979,7 @@ int pcg_run(int f32, const PcgLane *one, const PcgLane *lanes_dev, int nlanes, i
     constexpr int kRunSteps = 64;
     for (int done = 0; done < steps; done += kRunSteps) {
         const int now = steps - done < kRunSteps ? steps - done : kRunSteps;
-        cudaError_t e;
+        int e;
         switch (k) {
         case 8: e = f32 ? pcg_run_k<float, 8>(one, lanes_dev, nlanes, blocks, stage_bytes, now, st)
                         : pcg_run_k<double, 8>(one, lanes_dev, nlanes, blocks, stage_bytes, now, st); break;
@@ -4010,7 +3991,7 @@ int pcg_run(int f32, const PcgLane *one, const PcgLane *lanes_dev, int nlanes, i
                          : pcg_run_k<double, 64>(one, lanes_dev, nlanes, blocks, stage_bytes, now, st); break;
         default: return MBL_ERR_ARG;
         }
-        if (e != cudaSuccess) return MBL_ERR_CUDA;
+        if (e != MBL_OK) return done == 0 || e != kTooLarge ? e : MBL_ERR_CUDA;
     }
     return MBL_OK;
 }
@@ -4046,8 +4027,9 @@ static cudaError_t pcg_step_k(const ChainParams &cp, uint32_t n, const T *dinv, 
     return cudaGetLastError();
 }
 
-// One PCG iteration of the widths and switches without a resident kernel, on A = (H - sigma)^2: t = (H - sigma)p, alpha; r -= alpha (H - sigma)t,
-// beta; w += alpha p, p = M^-1 r + beta p.  Three launches, no host synchronisation.
+// One PCG iteration of the widths, sizes and switches without a resident kernel, on A =
+// (H - sigma)^2: t = (H - sigma)p, alpha; r -= alpha (H - sigma)t, beta; w += alpha p,
+// p = M^-1 r + beta p.  Three launches, no host synchronisation.
 template <typename T>
 int pcg_step(const ChainParams &cp, uint32_t n, int k, const T *dinv, T *r, T *p, T *t, T *w, const PcgDev &pd,
              cudaStream_t st)

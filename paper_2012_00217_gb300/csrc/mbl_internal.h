@@ -57,10 +57,16 @@ int pcg_start(const double *B, int64_t ldb, const double *bnorm, uint32_t n, int
 template <typename T>
 int pcg_step(const ChainParams &cp, uint32_t n, int k, const T *dinv, T *r, T *p, T *t, T *w, const PcgDev &pd,
              cudaStream_t st);
+// A cooperative launch of `blocks` blocks that wait for one another: kTooLarge (nothing launched)
+// where they do not fit on the SMs that the context has, a part of the device's.
+constexpr int kTooLarge = 1;
+int cooperative_launch(const void *kernel, unsigned blocks, unsigned threads, size_t smem, void **args,
+                       cudaStream_t st);
 // Resident PCG: `steps` PCG steps of one problem (`one`, lanes_dev null) or of nlanes
 // problems (lanes_dev: a device copy of PcgLane entries filled by pcg_lane_fill, in block
 // order), all of block width k with FP32 (f32) or FP64 vectors, in cooperative launches of
-// `blocks` blocks (the lanes' blocks together, at most one per SM).  may_stage: whole tiles
+// `blocks` blocks (the lanes' blocks together, at most one per SM); kTooLarge: not launched, for
+// pcg_step to do.  may_stage: whole tiles
 // through shared memory where the product's rule says so (a launch of one lane; stage_bytes
 // is then the lane's).  pcg_lane_passes: a lane's product work, to share blocks out by.
 struct PcgLane;
@@ -69,7 +75,8 @@ uint64_t pcg_lane_passes(int L, int n_up, int k, int f32);
 int pcg_lane_fill(PcgLane *lane, const ChainParams &cp, uint32_t n, int k, int f32, const void *dinv, void *r,
                   void *p, void *t, void *w, const PcgDev &pd, uint32_t block0, uint32_t max_blocks, bool may_stage);
 // Resident Lanczos steps j0 .. j0 + steps - 1 in one cooperative launch (mbl_apply.cu says
-// which vector is which); partials: >= 2 max_blocks doubles, counter: four zeroed words.
+// which vector is which); partials: >= 2 max_blocks doubles, counter: four zeroed words;
+// kTooLarge as above.
 bool lanczos_run_supported(int L, int n_up);
 int lanczos_run(const ChainParams &cp, uint32_t n, double *u, double *next, double *up, double *alpha, double *beta,
                 double *norm0, double *partials, unsigned *counter, uint32_t max_blocks, int j0, int steps,

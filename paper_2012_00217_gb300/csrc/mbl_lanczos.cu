@@ -218,7 +218,7 @@ int lanczos_bounds(const ChainParams &cp, int64_t n, const double *X0, int64_t l
     // v_0 = X0[:, 0] / ||X0[:, 0]||;  v_prev = 0
     note_launch();
     k_lz_start<<<grid, kLzThreads, 0, st>>>(X0, ldx0, d.v[1], n, nrm0, d.part, d.counter);
-    const bool resident = lanczos_run_supported(cp.L, cp.n_up);
+    bool resident = lanczos_run_supported(cp.L, cp.n_up);
     if (!resident) {
         note_launch();
         k_lz_scale<<<grid, kLzThreads, 0, st>>>(d.v[1], n, nrm0);
@@ -235,7 +235,13 @@ int lanczos_bounds(const ChainParams &cp, int64_t n, const double *X0, int64_t l
         if (resident) {
             const int rc = lanczos_run(cp, (uint32_t)n, d.v[iv], d.v[iw], d.v[ip], d.alpha, d.beta, nrm0, d.part,
                                        d.counter, (uint32_t)max_blocks, m, steps, st);
-            if (rc != MBL_OK) return rc;
+            if (rc == kTooLarge && m == 0) {  // the launches instead, on vectors of unit size
+                resident = false;
+                note_launch();
+                k_lz_scale<<<grid, kLzThreads, 0, st>>>(d.v[1], n, nrm0);
+            } else if (rc != MBL_OK) {
+                return rc < 0 ? rc : MBL_ERR_CUDA;
+            }
         }
         for (int j = m; j < m + steps; ++j) {
             if (!resident) {

@@ -169,6 +169,7 @@ struct Solver {
     Buffers b;
     cudaStream_t st;
     int64_t matvecs = 0;
+    bool resident = true;  // false once a cooperative launch did not fit: the PCG's own launches then
     // optional phase timing: events recorded at the phase boundaries of each iteration
     bool timing = false;
     cudaEvent_t ev[10] = {};
@@ -278,11 +279,13 @@ struct Solver {
     int enqueue_pcg_steps()
     {
         const PcgDev pd = pcg_dev();
-        if (pcg_run_supported(cp.L, cp.n_up, k, mixed)) {
+        if (resident && pcg_run_supported(cp.L, cp.n_up, k, mixed)) {
             PcgLane lane;
             MBL_TRY(pcg_lane_fill(&lane, cp, (uint32_t)n, k, mixed, b.dinv, b.pr, b.pp, b.pt, b.pw, pd, 0,
                                   (uint32_t)num_sms(), true));
-            return pcg_run(mixed, &lane, nullptr, 1, k, lane.nblocks, lane.stage_bytes, m, st);
+            const int rc = pcg_run(mixed, &lane, nullptr, 1, k, lane.nblocks, lane.stage_bytes, m, st);
+            if (rc != kTooLarge) return rc;
+            resident = false;
         }
         for (int it = 0; it < m; ++it) {
             if (mixed)
@@ -414,7 +417,8 @@ int run_body(Solver &s, bool have_p, bool use_graph, GraphCache &gc)
 {
     if (!use_graph) return s.enqueue_body(have_p);
     const int slot = have_p ? 1 : 0;
-    if (!gc.exec[slot]) {
+    while (!gc.exec[slot]) {
+        const bool resident = s.resident;
         if (!gc.cap && cudaStreamCreateWithFlags(&gc.cap, cudaStreamNonBlocking) != cudaSuccess) return MBL_ERR_CUDA;
         cudaStream_t user = s.st;
         s.st = gc.cap;
@@ -430,11 +434,15 @@ int run_body(Solver &s, bool have_p, bool use_graph, GraphCache &gc)
         set_capturing(false);
         s.st = user;
         s.matvecs = mv;  // counted again at each replay below
-        if (rc != MBL_OK) {
+        if (rc != MBL_OK || ce != cudaSuccess || !g) {
             if (g) cudaGraphDestroy(g);
-            return rc;
+            if (resident && !s.resident) {  // a launch that did not fit may end a capture: once more without
+                (void)cudaGetLastError();
+                continue;
+            }
+            return rc != MBL_OK ? rc : MBL_ERR_CUDA;
         }
-        if (ce != cudaSuccess || !g) return MBL_ERR_CUDA;
+        gc.kernels[slot] = 0;
         size_t nn = 0;
         if (cudaGraphGetNodes(g, nullptr, &nn) == cudaSuccess && nn > 0) {
             std::vector<cudaGraphNode_t> nodes(nn);
@@ -447,13 +455,26 @@ int run_body(Solver &s, bool have_p, bool use_graph, GraphCache &gc)
         }
         ce = cudaGraphInstantiate(&gc.exec[slot], g, 0);
         cudaGraphDestroy(g);
+        if (ce == cudaErrorCooperativeLaunchTooLarge && s.resident) {
+            (void)cudaGetLastError();
+            gc.exec[slot] = nullptr;
+            s.resident = false;
+            continue;
+        }
         if (ce != cudaSuccess) return MBL_ERR_CUDA;
     }
+    const cudaError_t le = cudaGraphLaunch(gc.exec[slot], s.st);
+    if (le == cudaErrorCooperativeLaunchTooLarge && s.resident) {
+        (void)cudaGetLastError();
+        s.resident = false;
+        gc.reset();
+        return run_body(s, have_p, use_graph, gc);
+    }
+    if (le != cudaSuccess) return MBL_ERR_CUDA;
+    note_launch(gc.kernels[slot]);
     // matvec accounting of one body
     s.matvecs += (int64_t)(s.folded ? 2 * s.m * s.k + 2 * s.k + (have_p ? 2 * s.k : 0) + 2 * s.k
                                     : s.k + (have_p ? s.k : 0) + s.k);
-    if (cudaGraphLaunch(gc.exec[slot], s.st) != cudaSuccess) return MBL_ERR_CUDA;
-    note_launch(gc.kernels[slot]);
     return MBL_OK;
 }
 
@@ -1010,6 +1031,7 @@ extern "C" int mbl_lobpcg_solve_batched(int nprob, const mbl_chain *chains, cons
     const bool graphs = opts->use_graph != 0;
     constexpr int kStallIters = 20;  // as in mbl_lobpcg_solve
     int next = 0, not_converged = 0;
+    bool shared = true;  // the lanes' PCG steps in shared cooperative launches
 
     // put problem next (if any) into lane l: its setup is enqueued now, its first status
     // is read in the next round
@@ -1129,10 +1151,11 @@ extern "C" int mbl_lobpcg_solve_batched(int nprob, const mbl_chain *chains, cons
         MBL_TRY(join());
         if (nb > 0 && opts->pcg_iters > 0) {
             // each advancing lane's share of the SMs, by its product work (at least one each);
-            // widths or switches without a resident kernel run each lane's own PCG launches
+            // widths or switches without a resident kernel, more lanes than SMs, and a context
+            // on whose SMs the shared launch does not fit run each lane's own PCG launches
             std::vector<int> in;
             std::vector<uint64_t> work;
-            bool fill = true;
+            bool fill = shared && nb <= num_sms();
             uint64_t total = 0;
             for (int l = 0; l < ns; ++l) {
                 if (!lanes[(size_t)l].body) continue;
@@ -1142,11 +1165,7 @@ extern "C" int mbl_lobpcg_solve_batched(int nprob, const mbl_chain *chains, cons
                 work.push_back(pcg_lane_passes(s.cp.L, s.cp.n_up, k, mixed));
                 total += work.back();
             }
-            if (!fill) {
-                MBL_TRY(fork());
-                for (int l : in) MBL_TRY(lanes[(size_t)l].s.enqueue_pcg_steps());
-                MBL_TRY(join());
-            } else {
+            if (fill) {
                 const int sms = num_sms();
                 std::vector<uint32_t> share(in.size());
                 int left = sms;
@@ -1172,7 +1191,14 @@ extern "C" int mbl_lobpcg_solve_batched(int nprob, const mbl_chain *chains, cons
                 if (cudaMemcpyAsync(table_dev, table.data(), sizeof(PcgLane) * in.size(), cudaMemcpyHostToDevice,
                                     st) != cudaSuccess)
                     return MBL_ERR_CUDA;
-                MBL_TRY(pcg_run(mixed, nullptr, table_dev, (int)in.size(), k, block0, 0, opts->pcg_iters, st));
+                const int prc = pcg_run(mixed, nullptr, table_dev, (int)in.size(), k, block0, 0, opts->pcg_iters, st);
+                if (prc == kTooLarge) fill = shared = false;
+                else MBL_TRY(prc);
+            }
+            if (!fill) {
+                MBL_TRY(fork());
+                for (int l : in) MBL_TRY(lanes[(size_t)l].s.enqueue_pcg_steps());
+                MBL_TRY(join());
             }
         }
         MBL_TRY(fork());
