@@ -1,6 +1,10 @@
 """The any-width product kernel against the oracle: widths with and without a divisor that makes a
-vector, wider than a warp's lanes, padded and misaligned blocks, off-centre sectors; and its stand-in
-under a capture that meets a tile width for the first time."""
+vector, wider than a warp's lanes, padded and misaligned blocks, off-centre sectors; and first products
+of a process under capture, and beside one."""
+import os
+import subprocess
+import sys
+
 import numpy as np
 import pytest
 
@@ -44,3 +48,49 @@ def test_any_width(mbl, dtype, L, n_up, periodic, k, ld, shift):
     got = ys[shift:].view(n, ld).cpu().numpy()
     assert np.all(got[:, k:] == 77.0) and torch.all(ys[:shift] == 77.0)
     assert np.all(np.abs(got[:, :k].astype(np.float64) - ref) <= _bound(chain, 0.4, Xb[:, :k], dtype))
+
+
+# A process whose first product of a tile width is captured (the any-width kernel's stand-in), or runs on
+# another stream while one is being captured; torch captures in the mode that forbids the most
+FIRST = """
+import sys
+import numpy as np, torch
+import paper_2012_00217_gb300 as mbl
+import workloads as wl
+from oracle import hamiltonian as ham
+L, k, beside = int(sys.argv[1]), int(sys.argv[2]), sys.argv[3] == "beside"
+n = ham.sector_dim(L, L // 2)
+h = wl.fields(L, 5.0, 1)
+Xb = wl.block(n, k, 2)
+ref = ham.apply(ham.Chain(L, h), 0.3, Xb)
+chain = mbl.make_chain(L, h)
+X = torch.from_numpy(Xb).cuda()
+Y, Z = torch.zeros_like(X), torch.zeros_like(X)
+other = torch.cuda.Stream()
+torch.cuda.synchronize()
+g = torch.cuda.CUDAGraph()
+with torch.cuda.graph(g):
+    if beside:
+        with torch.cuda.stream(other):
+            mbl.hamiltonian_apply(chain, 0.3, X, Z)
+        Y.add_(X)
+    else:
+        mbl.hamiltonian_apply(chain, 0.3, X, Y)
+other.synchronize()
+for _ in range(2):
+    Y.zero_()
+    g.replay()
+torch.cuda.synchronize()
+assert np.abs((Z if beside else Y).cpu().numpy() - ref).max() <= 1e-11
+if beside:
+    assert torch.equal(X, Y)
+print("agrees")
+"""
+
+
+@pytest.mark.parametrize("where", ["captured", "beside"])
+@pytest.mark.parametrize("L,k", [(10, 20), (10, 32), (16, 20), (16, 32)])
+def test_first_product_and_captures(mbl, L, k, where):
+    r = subprocess.run([sys.executable, "-c", FIRST, str(L), str(k), where], capture_output=True, text=True, timeout=300,
+                       cwd=os.path.dirname(os.path.dirname(os.path.abspath(__file__))))
+    assert r.returncode == 0 and "agrees" in r.stdout, r.stderr[-2000:]

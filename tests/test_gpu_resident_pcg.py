@@ -49,6 +49,30 @@ def test_solve_matches_dense(mbl, L, n_up, periodic, k, mode, pcg_iters, pcg_tol
     assert np.array_equal(again, evals)  # every sum has a fixed order
 
 
+# whole tiles through shared memory, by the switch: every width and type, rows below 128 bytes (whose
+# records stay in global memory) and above, more tiles than the groups have cached jobs for, one block
+@pytest.mark.parametrize("mode", [0, 1])
+@pytest.mark.parametrize("L,n_up,periodic,k,nev", [
+    (12, 6, True, 8, 4), (13, 5, False, 8, 4), (12, 6, False, 16, 8), (12, 6, True, 32, 16), (12, 7, False, 64, 32),
+    (8, 4, True, 16, 8), (14, 7, False, 64, 16)])
+def test_staged_solve_matches_dense(mbl, L, n_up, periodic, k, nev, mode):
+    h = wl.fields(L, 6.0, 80 + L)
+    ev = np.linalg.eigvalsh(ham.dense_sector(ham.Chain(L, h, n_up=n_up, periodic=periodic)))
+    sigma, norm_h = 0.5 * (ev[0] + ev[-1]), max(abs(ev[0]), abs(ev[-1]))
+    want = np.sort(ev[np.lexsort((ev, np.abs(ev - sigma)))[:nev]])
+    try:
+        for t in (torch.float32, torch.float64):
+            mbl.binding.set_product_schedule(k, t, 3)
+        evals, resid, stats, _ = _solve(mbl, L, n_up, h, periodic, sigma, nev, k, mode, norm_h, 40)
+        again, _, _, _ = _solve(mbl, L, n_up, h, periodic, sigma, nev, k, mode, norm_h, 40)
+    finally:
+        for t in (torch.float32, torch.float64):
+            mbl.binding.set_product_schedule(k, t, 0)
+    assert stats["converged"] == 1 and resid.max() <= 1e-8 * norm_h
+    assert np.abs(evals - want).max() <= (1e-6 if mode else 1e-9) * norm_h
+    assert np.array_equal(again, evals)
+
+
 def test_batch_with_w_outside_tensor_memory(mbl):
     """64 lanes on the SMs leave a lane of 3,432 rows two blocks, 1,716 rows each: more than the
     1,008 rows of 32 FP64 columns that a block's tensor memory holds.  The single solve (23
