@@ -105,14 +105,16 @@ __device__ __forceinline__ bool jacobi_rotation(double apq, double app, double a
 // with |a_pq| <= eps sqrt(|a_pp a_qq|) are skipped (the relative test keeps the small
 // eigenvalues of graded matrices accurate); sweeps stop when one rotates nothing or after
 // max_sweeps.  On exit diag(A) holds the eigenvalues and the columns of V (stride ld)
-// the eigenvectors.  Each warp rotates whole rows / columns of its pairs, lanes striding the other index.  cs, pairs: n + 2
+// the eigenvectors (WANT_V = false: eigenvalues only, V not touched).  Each warp rotates
+// whole rows / columns of its pairs, lanes striding the other index.  cs, pairs: n + 2
 // entries (shared or global memory of this block).
-template <typename T>
+template <typename T, bool WANT_V = true>
 __device__ void dev_jacobi(int n, int ld, T *A, T *V, T *cs, int *pairs, int *s_rot, int max_sweeps)
 {
     const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5, nwarps = nt >> 5;
-    for (int i = warp; i < n; i += nwarps)
-        for (int j = lane; j < n; j += 32) V[i * ld + j] = (i == j) ? (T)1 : (T)0;
+    if (WANT_V)
+        for (int i = warp; i < n; i += nwarps)
+            for (int j = lane; j < n; j += 32) V[i * ld + j] = (i == j) ? (T)1 : (T)0;
     __syncthreads();
     if (n < 2) return;
     const int np = (n + 1) & ~1;
@@ -165,10 +167,12 @@ __device__ void dev_jacobi(int n, int ld, T *A, T *V, T *cs, int *pairs, int *s_
                     const T ap = Aj[p], aq = Aj[q];
                     Aj[p] = c * ap - s * aq;
                     Aj[q] = s * ap + c * aq;
-                    T *Vj = V + j * ld;
-                    const T vp = Vj[p], vq = Vj[q];
-                    Vj[p] = c * vp - s * vq;
-                    Vj[q] = s * vp + c * vq;
+                    if (WANT_V) {
+                        T *Vj = V + j * ld;
+                        const T vp = Vj[p], vq = Vj[q];
+                        Vj[p] = c * vp - s * vq;
+                        Vj[q] = s * vp + c * vq;
+                    }
                 }
             }
             __syncthreads();
@@ -702,10 +706,12 @@ int gather_cols(int k, int nev, const double *V, const int *sel, double *Csel, c
 //   k_ent_eig      its eigenvalues by bisection on Sturm counts, one lane each, and the
 //                  sum of lambda ln lambda;
 // and k_ent_combine forms S = ln N - (sum lambda ln lambda) / N with N = sum lambda, the
-// trace of the Grams, so v need not be normalised.  Every sum has a fixed order.
+// trace of the Grams, so v need not be normalised.  Every sum has a fixed order.  Eigenvalues
+// are absolute to 2^-60 of the trace (their share of S to 1e-14).  Cuts of small Grams take
+// k_ent_block instead (ent_one_block).
 //
 // All of it is bound by the FP64 pipe (two FMA a cycle and SM on GB300).  At L = 20,
-// l_a = 10, 16 vectors, the one-block FP64 Jacobi in L2 that this replaces took 590 ms,
+// l_a = 10, 16 vectors, the one-block FP64 Jacobi in L2 (k_ent_block) took 590 ms,
 // about 20 sweeps of n^3 rotations; the reduction needs n^3 FMA once, spread over four SMs
 // a matrix (6.7 ms the whole call).
 
@@ -1061,6 +1067,115 @@ __global__ void k_ent_combine(EntCut cut, int nvec, double *work, double *S)
     S[e] = n2 > 0.0 ? log(n2) - a1 / n2 : NAN;
 }
 
+// The whole of one (vector, p) in one block, and the sums over p: for cuts whose Grams are small
+// or long sums.
+__global__ void __launch_bounds__(kSmallThreads)
+    k_ent_block(int L, int n_up, int la, const double *__restrict__ V, int64_t ldv, double *work,
+                int64_t block_doubles, int64_t mmax, int64_t dmax, double *parts)
+{
+    __shared__ uint32_t sb[kBinomDim * kBinomDim];
+    __shared__ int s_rot;
+    __shared__ double s_r0[kSmallThreads / 32], s_r1[kSmallThreads / 32];
+    load_binom(sb);
+    __syncthreads();
+    const int e = blockIdx.x / (la + 1), p = blockIdx.x % (la + 1);
+    const int lb = L - la, q = n_up - p;
+    double *out = parts + 2 * (int64_t)blockIdx.x;
+    if (q < 0 || q > lb) {  // no state has p up spins on the left
+        if (threadIdx.x == 0) {
+            out[0] = 0.0;
+            out[1] = 0.0;
+        }
+        return;
+    }
+    const int R = (int)binom(sb, la, p), T = (int)binom(sb, lb, q);
+    const bool left = R <= T;  // Gram over the left patterns (d = R), else over the right ones
+    const int d = left ? R : T, ld = pad_ld(d);
+    double *M = work + (int64_t)blockIdx.x * block_doubles;  // R x T, row-major
+    double *A = M + mmax;
+    double *cs = A + dmax * (int64_t)pad_ld((int)dmax);
+    int *pairs = reinterpret_cast<int *>(cs + dmax + 2);
+    uint32_t *off = reinterpret_cast<uint32_t *>(cs + 2 * (dmax + 2));
+    for (int c = threadIdx.x; c < T; c += blockDim.x) {
+        const uint32_t b = cns_unrank(sb, lb, q, (uint32_t)c);
+        off[c] = cns_rank(sb, (b << la) | ((1u << p) - 1u));
+    }
+    __syncthreads();
+    const double *v = V + e;
+    for (int64_t x = threadIdx.x; x < (int64_t)R * T; x += blockDim.x) {
+        const int i = (int)(x % R), c = (int)(x / R);  // consecutive threads: consecutive rows of a tile
+        M[(int64_t)i * T + c] = v[((int64_t)off[c] + i) * ldv];
+    }
+    __syncthreads();
+    for (int64_t x = threadIdx.x; x < (int64_t)d * d; x += blockDim.x) {
+        const int i = (int)(x / d), j = (int)(x % d);
+        if (j < i) continue;
+        double acc = 0.0;
+        if (left) {
+            const double *mi = M + (int64_t)i * T, *mj = M + (int64_t)j * T;
+            for (int c = 0; c < T; ++c) acc += mi[c] * mj[c];
+        } else {
+            for (int r = 0; r < R; ++r) acc += M[(int64_t)r * T + i] * M[(int64_t)r * T + j];
+        }
+        A[(int64_t)i * ld + j] = acc;
+        A[(int64_t)j * ld + i] = acc;
+    }
+    __syncthreads();
+    dev_jacobi<double, false>(d, ld, A, nullptr, cs, pairs, &s_rot, kMaxSweeps);
+    double s0 = 0.0, s1 = 0.0;
+    for (int i = threadIdx.x; i < d; i += blockDim.x) {
+        const double lam = A[(int64_t)i * ld + i];
+        if (!(lam <= 0.0)) {  // NaN too: an entry that is not finite makes S NaN
+            s0 += lam;
+            s1 += lam * log(lam);
+        }
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+        s0 += __shfl_xor_sync(0xffffffffu, s0, o);
+        s1 += __shfl_xor_sync(0xffffffffu, s1, o);
+    }
+    if ((threadIdx.x & 31) == 0) {
+        s_r0[threadIdx.x >> 5] = s0;
+        s_r1[threadIdx.x >> 5] = s1;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        double a0 = 0.0, a1 = 0.0;
+        for (int w = 0; w < kSmallThreads / 32; ++w) {
+            a0 += s_r0[w];
+            a1 += s_r1[w];
+        }
+        out[0] = a0;
+        out[1] = a1;
+    }
+}
+
+__global__ void k_ent_block_combine(int nvec, int per, const double *parts, double *S)
+{
+    const int e = blockIdx.x * blockDim.x + threadIdx.x;
+    if (e >= nvec) return;
+    double n2 = 0.0, a1 = 0.0;
+    for (int p = 0; p < per; ++p) {
+        n2 += parts[2 * ((int64_t)e * per + p)];
+        a1 += parts[2 * ((int64_t)e * per + p) + 1];
+    }
+    S[e] = n2 > 0.0 ? log(n2) - a1 / n2 : NAN;
+}
+
+// Whether a cut takes k_ent_block: Grams of side 4 and less, or 6 for few vectors, whose four
+// kernels are all launches, and those with sums over more than d^3 / 4 entries, which k_ent_gram
+// forms for the whole of a 32 x 32 tile.  us, k_ent_block / the kernels above: d = 4, t = 15, 16
+// vectors 62 / 95;  d = 6, t = 20, 1 vector 95 / 116, 200 vectors 225 / 200;  16 vectors, d = 6,
+// t = 210 128 / 177;  d = 10, t = 126 241 / 197, t = 462 250 / 297, t = 6435 485 / 2106;  d = 20,
+// t = 924 723 / 565, t = 3432 728 / 1318;  d = 35, t = 1716 2608 / 1352.
+static bool ent_one_block(int L, int n_up, int la, int nvec, int64_t d)
+{
+    int64_t t = 0;
+    for (int p = std::max(0, n_up - (L - la)); p <= std::min(la, n_up); ++p)
+        t = std::max<int64_t>(t, std::max(host_binom(la, p), host_binom(L - la, n_up - p)));
+    return d <= 4 || (d <= 6 && nvec <= 8) || 4 * t > d * d * d;
+}
+
 int entanglement_launch(int L, int n_up, int la, int nvec, const double *V, int64_t ldv, double *S, void *work,
                         size_t work_bytes, cudaStream_t st)
 {
@@ -1068,6 +1183,17 @@ int entanglement_launch(int L, int n_up, int la, int nvec, const double *V, int6
     const size_t need = entanglement_work_bytes(pl, nvec);
     if (work_bytes < need) return MBL_ERR_WORKSPACE;
     double *w = (double *)(((uintptr_t)work + 255) & ~(uintptr_t)255);
+    if (ent_one_block(L, n_up, la, nvec, pl.dmax)) {
+        const int64_t nblk = (int64_t)nvec * pl.blocks_per_vector;
+        double *parts = w + nblk * pl.block_doubles;
+        note_launch();
+        k_ent_block<<<(unsigned)nblk, kSmallThreads, 0, st>>>(L, n_up, la, V, ldv, w, pl.block_doubles, pl.mmax, pl.dmax,
+                                                              parts);
+        if (cudaGetLastError() != cudaSuccess) return MBL_ERR_CUDA;
+        note_launch();
+        k_ent_block_combine<<<(nvec + 127) / 128, 128, 0, st>>>(nvec, pl.blocks_per_vector, parts, S);
+        return cudaGetLastError() == cudaSuccess ? MBL_OK : MBL_ERR_CUDA;
+    }
     EntCut cut{};
     cut.L = L;
     cut.n_up = n_up;

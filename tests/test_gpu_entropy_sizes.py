@@ -60,3 +60,22 @@ def test_not_finite_and_many_columns(mbl):
     assert math.isnan(S[7]) and math.isnan(S[8])
     for e in (0, 6, 9, 4500, 8999):
         assert abs(S[e] - obs.entanglement_entropy(st, V[:, e], 4)) <= 1e-10
+
+
+# cuts of small Grams and long sums, one kernel and its combine (2 launches), beside the five kernels
+@pytest.mark.parametrize("L,n_up,l_a,launches", [
+    (8, 4, 2, 2), (10, 5, 3, 2), (14, 7, 3, 2), (16, 8, 4, 2), (18, 9, 4, 2), (20, 10, 5, 2), (20, 10, 16, 2), (12, 1, 6, 2), (20, 7, 6, 2), (10, 5, 4, 2),
+    (10, 5, 5, 5), (12, 6, 5, 5), (14, 7, 7, 5), (18, 9, 7, 5)])
+def test_small_grams(mbl, L, n_up, l_a, launches):
+    rng = np.random.default_rng(L * 17 + l_a)
+    st = ham.basis(L, n_up)
+    V = _columns(L, st, rng)
+    V = np.concatenate([V, np.zeros((st.size, 2))], axis=1)
+    V[st.size // 2, 5] = np.nan
+    chain = mbl.make_chain(L, np.zeros(L), 1.0, False, n_up)
+    before = mbl.binding.kernel_launch_count()
+    S = mbl.entanglement_entropy(chain, l_a, torch.from_numpy(V.copy()).to(DEV)).cpu().numpy()
+    assert mbl.binding.kernel_launch_count() - before == launches
+    for e in range(4):
+        assert abs(S[e] - obs.entanglement_entropy(st, V[:, e], l_a)) <= 1e-10, e
+    assert math.isnan(S[4]) and math.isnan(S[5])  # a zero column, a NaN
