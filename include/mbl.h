@@ -304,11 +304,12 @@ int mbl_lobpcg_solve_noalloc(const mbl_chain *chain, double sigma, const mbl_lob
  * the steps before and after the preconditioner are enqueued lane by lane, and the
  * pcg_iters PCG steps of all advancing lanes run in cooperative launches of up to 64 steps,
  * every lane on its own share of the SMs (where such a launch does not fit, in a context
- * that has a part of the device's SMs, every lane runs its own launches of single steps).  When a lane's problem converges (or reaches max_iter) its results are
- * written and it takes the next problem.  The host synchronises `stream` once per round
- * to read the lanes' status words.  With opts->use_graph, each lane's steps before and
- * after the preconditioner are captured once per problem as two small CUDA graphs and
- * replayed every round; opts->timing is ignored (use_graph = 0 with timing = 1 is
+ * that has a part of the device's SMs, every lane runs its own launches of single steps).
+ * When a lane's problem converges (or reaches max_iter) its results are written and it
+ * takes the next problem.  The host synchronises `stream` once per round to read the
+ * lanes' status words.  With opts->use_graph, each lane's steps before and after the
+ * preconditioner are captured once per problem as two small CUDA graphs and replayed
+ * every round; opts->timing is ignored (use_graph = 0 with timing = 1 is
  * MBL_ERR_ARG).  Every problem's results equal the single-problem solve's to within
  * rounding (the PCG of a lane runs the same arithmetic on fewer SMs; widths k other than 8,
  * 16, 32, 64, and lanes whose four PCG vectors exceed 100 MB, run each lane's own PCG
@@ -375,8 +376,9 @@ int mbl_gap_ratio(int nprob, int m, const double *evals_dev, int64_t ld, double 
  * is the direct sum over p (up spins on the left) of M_p M_p^T, M_p holding the column's
  * entries with p up spins on the left (rows: left patterns, columns: right patterns); its
  * eigenvalues come from the smaller Gram of each M_p, in FP64 (Householder reduction and
- * bisection).  Writes S_dev[nvec]
- * (FP64 device memory; NaN for a zero column).  chain->h, delta and periodic are not used.
+ * bisection, to 2^-60 of the trace; Jacobi for small Grams).  Writes S_dev[nvec]
+ * (FP64 device memory; NaN for a zero column and one that is not finite).  chain->h, delta
+ * and periodic are not used.
  * Limit: every Gram side min(C(l_a, p), C(L - l_a, n_up - p)) <= 512 (the half cut up to
  * L = 22), else MBL_ERR_ARG.  Workspace: mbl_entanglement_workspace_size bytes of device
  * memory (about 1 MB per column and p at L = 20, l_a = 10).  Deterministic (fixed-order

@@ -602,7 +602,8 @@ __device__ __forceinline__ const LowRec *low_table(int B, int k)
 }
 
 // Resident blocks per SM the tiled kernel is compiled for (register budget 65536 /
-// (256 * this)); 3 keeps every variant free of spills.
+// (256 * this)), 3: 80 registers.  Lanes of 16 and 32 bytes fit in plain products; 64-byte
+// lanes spill 72 to 96 bytes there, and the PCG launches 8 to 390.
 #ifndef MBL_TILED_MIN_BLOCKS
 #define MBL_TILED_MIN_BLOCKS 3
 #endif
@@ -1052,7 +1053,7 @@ __device__ __forceinline__ void fence_proxy_async_smem() { asm volatile("fence.p
 // Whether the staged kernels copy a tile's records beside its rows: for rows of at least 128
 // bytes, where they add a quarter at most.  A row's gathers wait for its record, and from
 // shared memory that is one L2 latency less in the chain of every row pass (L = 20, k = 32,
-// FP32: product 28.8 -> 28.2 us, PCG step 82.9 -> 82.2 us).
+// FP32: 0.6 us less a product, 0.7 us a PCG step).
 template <typename T, int K>
 __host__ __device__ constexpr bool stage_records()
 {
@@ -2204,13 +2205,14 @@ __global__ void __launch_bounds__(kThreads) k_pcg_update(uint32_t n, const T *__
 // through that order there and back (staged), or cut into row chunks dealt out to the warps.
 // Every block sums all partials of its lane itself, in a fixed order, right after the
 // barrier.  Measured (GB300, us a step, three launches -> resident):
-//   FP32  L = 12, k = 8: 32.8 -> 13.9;  16, 16: 40.3 -> 16.4;  18, 32: 53.1 -> 29.3;
-//         20, 32: 97.4 -> 77.5
-//   FP64  L = 14, k = 16: 118 -> 44;  18, 32: 236 -> 164
-// At L = 20, k = 32 the phases take about 22, 27 and 11 us, bound by L2 gathers and streams
-// at the loads a block has in flight, and the three barriers with their sums the rest.
-// Beyond L2 (a lane's four vectors above 100 MB) the launches are as fast or faster (L = 20,
-// k = 64: 185 against 190 us; L = 22, k = 32: 301 against 404 us) and stay.
+//   FP32  L = 12, k = 8: 32.8 -> 14.2;  16, 16: 40.3 -> 16.4;  18, 32: 53.1 -> 29.0;
+//         20, 32: 97.4 -> 78.4
+//   FP64  L = 14, k = 16: 118 -> 42.8;  18, 32: 236 -> 162
+// At L = 20, k = 32 the phases take 20.7, 22.7 and 11.4 us (means over the blocks; the slowest
+// block 24.5, 26.5 and 14.4), bound by L2 gathers and streams at the loads a block has in
+// flight; the barriers, their sums and the wait for the slowest block take the other 23.5.
+// Beyond L2 (a lane's four vectors above 100 MB) the launches are faster (L = 20, k = 64: 169
+// against 190 us; L = 22, k = 32: 291 against 404 us) and stay.
 //
 // A lane's blocks wait for one another, so the launch is cooperative.  Every wait is
 // bounded; on a time-out, of a barrier or of a staged copy, the lane's fail word is set.  The
@@ -2259,7 +2261,8 @@ struct ColSum<float> {
     __device__ __forceinline__ bool positive() const { return s > 0.0f && isfinite(s) && isfinite(e); }
     __device__ __forceinline__ bool finite() const { return isfinite(s) && isfinite(e); }
     // (s + e) / (d.s + d.e) in FP32: the quotient of the leading parts and one correction by
-    // the remainder, which the fma gives exactly; within an ulp of the rounded FP64 quotient
+    // the remainder, which the fma gives exactly: within half an ulp and 1e-6 of the exact one,
+    // as the FP64 quotient rounded to FP32
     __device__ __forceinline__ float over(const ColSum &d) const
     {
         const float q = s / d.s;
@@ -2521,7 +2524,7 @@ __device__ __forceinline__ bool group_all(int id, bool mine)
 // y.y (kPcgT) or x.y (kDot), or q = (H - sigma) X, R -= alpha q and the sum of R.(M^-1 R)
 // (kPcgQ), into sm.red.  Staged: a group of 256 threads takes whole tiles, one at a time: the other groups
 // work while its copy is in flight, and a second buffer would come out of the L1 that loads
-// in flight need (L = 20, k = 32: 105 us a step with two buffers, 93 with one).  Else a
+// in flight need (L = 20, k = 32: a second one made a step 13 % slower).  Else a
 // warp takes a chunk of a tile.
 template <typename T, int K, int MODE, bool STAGED>
 __device__ __noinline__ void run_product()
@@ -2684,10 +2687,10 @@ __device__ __forceinline__ void run_move_w(uint32_t row_b, uint32_t row_e, uint3
 
 // w += alpha p, p = M^-1 r + beta p for rows [row_b, row_e), the block's share.  W_TMEM: w
 // stays in tensor memory for the whole launch, which takes two of the phase's five vector
-// streams off L2 (L = 20, k = 32: 25 -> 18 us for this phase).  A row a thread at a time and
-// inlined: more rows in flight cost more in saved and spilled registers than they gave (a
-// step at L = 20, k = 32: 91 us with seven rows, 82.4 with three, 78.8 with one, and 77.5
-// with the sums a function of their own instead).
+// streams off L2 (L = 20, k = 32: 7 us of this phase).  A row a thread at a time and inlined:
+// more rows in flight cost more in saved and spilled registers than they gave (a step at
+// L = 20, k = 32: 12 us more with seven rows, 4 with three; 1 less with the sums a function of
+// their own instead).
 template <typename T, int K, bool W_TMEM>
 __device__ __forceinline__ void run_update(uint32_t row_b, uint32_t row_e, uint32_t tmem)
 {

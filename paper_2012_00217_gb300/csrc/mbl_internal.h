@@ -12,7 +12,8 @@ namespace mbl {
 struct ChainParams;
 
 // Device-resident per-column PCG state plus the block-partials scratch used by the
-// deterministic reductions (partials: >= grid * 64 doubles; counter: one zeroed word).
+// deterministic reductions (partials: >= grid * 64 doubles; counter: four zeroed words, the
+// first the launches' ticket, the others the resident kernel's).
 struct PcgDev {
     double *rz, *rz0, *alpha, *beta;
     int *active;
