@@ -3176,10 +3176,9 @@ static int kslot(int K)
 
 uint32_t host_binom(int n, int k)
 {
-    if (k < 0 || k > n) return 0;
-    uint64_t c = 1;
-    for (int i = 1; i <= k; ++i) c = c * (uint64_t)(n - k + i) / (uint64_t)i;
-    return (uint32_t)c;
+    // the rules of a product's dispatch ask about ten times a call
+    static constexpr BinomTable table = make_binom_table();
+    return k < 0 || k > n ? 0 : table.v[n * kBinomDim + k];
 }
 
 // Tile width heuristic: the widest table-backed tiles (B = 13, at most L - 2 so that two
@@ -3257,8 +3256,8 @@ static int size_schedule(int L, int n_up, int K, size_t es)
     if (row >= 256 && mb >= 1024.0) return 2;
     if (row == 128) return mb >= 16.0 ? 3 : 1;
     const int B = heuristic_tile_bits(L, K, es);
-    if ((row != 64 && row != 256) || B < 2 || tile_fill(L, n_up, B) < 0.6) return 1;
-    return mb >= (row == 256 ? 32.0 : 16.0) ? 3 : 1;
+    if ((row != 64 && row != 256) || mb < (row == 256 ? 32.0 : 16.0) || B < 2) return 1;
+    return tile_fill(L, n_up, B) >= 0.6 ? 3 : 1;
 }
 
 static int explicit_schedule(int K, size_t es) { return g_schedule[es == 8 ? 1 : 0][kslot(K)]; }
